@@ -979,3 +979,33 @@ def test_general_sorted_w_matches_oracle(p):
         tk.tk_fwd_w(th, wt, 4, 1024, 1.5, 1.0, o)
     assert e.value.status == tk.TK_ERR_UNSUPPORTED
 
+
+
+@pytest.mark.parametrize("n", [1, 2, 8, 9, 15, 16, 17, 32, 33, 65, 256, 257, 512, 513, 1024, 1025, 2047, 2048])
+def test_general_sorted_w_exact_ties_at_team_edges(n):
+    """tk_fwd_w / tk_vjp_w around every change of the row's team (8 or 16 ranks per lane), on data whose block sums
+    are exact in any order (multiples of 1/8, lambda = 1, p = 2): long runs of equal keys and of equal w, so
+    the partition and the stable order inside a run are determined and every element must match the oracle.
+    Few rows (8 ranks per lane) and, for short rows, enough of them for 16."""
+    from oracle import tko
+    rng = np.random.Generator(np.random.PCG64(4000 + n))
+    for rows in (21 if n <= 512 else 5, (1 << 20) // n + 3 if n <= 33 else 6):
+        x = (rng.integers(-24, 25, (rows, n)) / 8.0).astype(np.float32)
+        x[0] = 0.5                                       # one run of equal keys
+        x[1] = np.sort(x[1])[::-1]
+        g = wl.cotangent_like(x, 4100 + n)
+        k = max(1, n // 3)
+        ones_k = np.r_[np.ones(k), np.zeros(n - k)].astype(np.float32)
+        levels = np.sort(rng.integers(-8, 9, (rows, n)) / 4.0, axis=1)[:, ::-1].astype(np.float32)
+        steep = (np.arange(n, 0, -1) / 8.0).astype(np.float32)          # pools almost everything
+        for label, w in (("1_k", ones_k), ("levels", levels), ("steep", steep)):
+            th, gt = torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda()
+            wt = torch.from_numpy(np.ascontiguousarray(w)).cuda()
+            out, grad, gw = (torch.full((rows, n), float("nan"), device="cuda") for _ in range(3))
+            tk.tk_fwd_w(th, wt, rows, n, 2.0, 1.0, out)
+            tk.tk_vjp_w(th, wt, gt, rows, n, 2.0, 1.0, grad, grad_w=gw)
+            torch.cuda.synchronize()
+            gref, gwref = tko.vjp_w(x, w, g, 2.0, 1.0, with_w=True)
+            for name, a, b in (("forward", out, tko.fwd_w(x, w, 2.0, 1.0)), ("vjp", grad, gref), ("vjp in w", gw, gwref)):
+                e = np.abs(a.cpu().numpy() - b) / np.maximum(1.0, np.abs(b))
+                assert e.max() <= 1e-5, f"{label} n={n} {name}: {e.max()} at {np.unravel_index(e.argmax(), e.shape)}"
