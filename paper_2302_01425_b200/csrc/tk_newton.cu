@@ -161,35 +161,6 @@ struct NtIO {
   }
 };
 
-// One key against the window (t = key - tau): capped (t >= width), inside (0 < t < width) or zero.
-// Counts and the inside keys' sums of t, t^2, t^3.
-template <bool Q4>
-__device__ __forceinline__ void nt_classify(float t, float wid, float& ct, float& cm, float& a, float& b, float& e) {
-  // two compares, then adds under their predicates (written out so that no select is formed)
-  if (!Q4) {
-    asm("{\n\t.reg .pred ptop, pmid;\n\t"
-        "setp.ge.f32 ptop, %3, %4;\n\t"
-        "setp.gt.and.f32 pmid, %3, 0f00000000, !ptop;\n\t"
-        "@ptop add.f32 %0, %0, 0f3F800000;\n\t"
-        "@pmid add.f32 %1, %1, 0f3F800000;\n\t"
-        "@pmid add.f32 %2, %2, %3;\n\t}"
-        : "+f"(ct), "+f"(cm), "+f"(a)
-        : "f"(t), "f"(wid));
-  } else {
-    asm("{\n\t.reg .pred ptop, pmid;\n\t.reg .f32 t2;\n\t"
-        "setp.ge.f32 ptop, %5, %6;\n\t"
-        "setp.gt.and.f32 pmid, %5, 0f00000000, !ptop;\n\t"
-        "mul.f32 t2, %5, %5;\n\t"
-        "@ptop add.f32 %0, %0, 0f3F800000;\n\t"
-        "@pmid add.f32 %1, %1, 0f3F800000;\n\t"
-        "@pmid add.f32 %2, %2, %5;\n\t"
-        "@pmid add.f32 %3, %3, t2;\n\t"
-        "@pmid fma.rn.f32 %4, t2, %5, %4;\n\t}"
-        : "+f"(ct), "+f"(cm), "+f"(a), "+f"(b), "+f"(e)
-        : "f"(t), "f"(wid));
-  }
-}
-
 // Keeps the loads of later chunks behind this point: the second passes over a row (new pivot, top-k
 // values, smallest capped key) run while the row's registers are live, and E more words in flight would spill.
 __device__ __forceinline__ void nt_fence() { asm volatile("" ::: "memory"); }

@@ -1009,3 +1009,33 @@ def test_general_sorted_w_exact_ties_at_team_edges(n):
             for name, a, b in (("forward", out, tko.fwd_w(x, w, 2.0, 1.0)), ("vjp", grad, gref), ("vjp in w", gw, gwref)):
                 e = np.abs(a.cpu().numpy() - b) / np.maximum(1.0, np.abs(b))
                 assert e.max() <= 1e-5, f"{label} n={n} {name}: {e.max()} at {np.unravel_index(e.argmax(), e.shape)}"
+
+
+@pytest.mark.parametrize("n", [2, 63, 64, 65, 128, 129, 1024, 1025, 2048, 2049, 4096, 4097])
+def test_slow_axis_at_the_edges_of_the_column_layouts(n):
+    """tk_fwd_cols / tk_vjp_cols around every change of the rows held per lane and of the warps per column, with a
+    ragged last group of 8 columns; the VJP reads the copy of theta the forward pass left, also when that pass
+    sorted (PAV, permutation) and the VJP's own kernels do not."""
+    from oracle import tko
+    from parity import rel_err, TOL
+    for cols, mode, p, solver in ((19, tk.TK_MASK, 2.0, tk.TK_SOLVER_AUTO), (8, tk.TK_TOPK, P43, tk.TK_SOLVER_PAV),
+                                  (9, tk.TK_TOPKMAG, 2.0, tk.TK_SOLVER_AUTO), (3, tk.TK_MASK, P43, tk.TK_SOLVER_AUTO),
+                                  (5, tk.TK_TOPKMAG, P43, tk.TK_SOLVER_AUTO)):
+        ld, k, lam = cols + 3, max(1, n // 6), 0.7
+        x, g = rows_of(n, ld, 7000 + n + cols, 1.0).T.copy(), rows_of(n, ld, 7500 + n + cols, 1.0).T.copy()
+        th, gt = torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda()
+        out, grad = torch.full_like(th, -7.0), torch.full_like(th, -7.0)
+        ws = torch.empty(tk.tk_cols_workspace_bytes(n, cols), dtype=torch.uint8, device="cuda")
+        state = tk.new_state(cols)
+        perm = torch.empty(cols, n, dtype=torch.int32, device="cuda") if solver == tk.TK_SOLVER_PAV else None
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        tk.tk_fwd_cols(th, n, cols, ld, k, p, lam, mode, out, workspace=ws, state_out=state, solver=solver,
+                       perm_out=perm, status_out=status)
+        tk.tk_vjp_cols(None, gt, n, cols, ld, k, p, lam, mode, grad, workspace=ws, state=state, status_out=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        xt, gtt = np.ascontiguousarray(x[:, :cols].T), np.ascontiguousarray(g[:, :cols].T)
+        o, gr = out.cpu().numpy(), grad.cpu().numpy()
+        assert rel_err(o[:, :cols], tko.fwd(xt, k, p, lam, mode).T).max() <= TOL, (n, cols, mode, p)
+        assert rel_err(gr[:, :cols], tko.vjp(xt, gtt, k, p, lam, mode).T).max() <= TOL, (n, cols, mode, p)
+        assert (o[:, cols:] == -7.0).all() and (gr[:, cols:] == -7.0).all()
