@@ -1039,3 +1039,28 @@ def test_slow_axis_at_the_edges_of_the_column_layouts(n):
         assert rel_err(o[:, :cols], tko.fwd(xt, k, p, lam, mode).T).max() <= TOL, (n, cols, mode, p)
         assert rel_err(gr[:, :cols], tko.vjp(xt, gtt, k, p, lam, mode).T).max() <= TOL, (n, cols, mode, p)
         assert (o[:, cols:] == -7.0).all() and (gr[:, cols:] == -7.0).all()
+
+
+@pytest.mark.parametrize("n", [1, 2, 16, 17, 64, 65, 128, 257, 512, 513, 1025, 2048, 2049, 4096])
+def test_sweeps_on_the_ranks_they_reach(n):
+    """The windowed sweeps against the oracle's sweeps over the whole row: every layout of the sorting team, windows
+    that touch either end of the row, one and several ranks per lane, runs of equal keys across the window's edges
+    (the permutation must be the stable one), the magnitude mode."""
+    from oracle import tko
+    from parity import rel_err
+    rows = 37 if n <= 128 else 5
+    for sweeps, k in ((1, 1), (3, max(1, n // 2)), (10, max(1, n // 9)), (100, max(1, n // 3)), (20, n)):
+        for mode, p in ((tk.TK_MASK, 2.0), (tk.TK_TOPKMAG, 2.0), (tk.TK_TOPK, P43)):
+            x = rows_of(n, rows, 8000 + n + sweeps, 1.0)
+            x[1] = np.round(x[1] * 4) / 4                           # runs of equal keys
+            x[2, :] = 0.25
+            th = torch.from_numpy(x).cuda()
+            out = torch.full_like(th, float("nan"))
+            perm = torch.empty(rows, n, dtype=torch.int32, device="cuda")
+            for want_perm in (False, True):
+                tk.tk_fwd_ex(th, rows, n, k, p, 0.7, mode, out, solver=tk.TK_SOLVER_DYKSTRA, sweeps=sweeps,
+                             perm_out=perm if want_perm else None)
+                torch.cuda.synchronize()
+                ref = tko.dykstra(x, k, p, 0.7, mode, sweeps=sweeps)
+                assert rel_err(out.cpu().numpy(), ref).max() <= 1e-5, (n, sweeps, k, mode, want_perm)
+            assert np.array_equal(perm.cpu().numpy(), tko.argsort(x, mode)[0]), (n, sweeps, mode)
