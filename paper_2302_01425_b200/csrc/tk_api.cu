@@ -29,6 +29,10 @@ cudaError_t launch_dykstra_cluster(const Problem& P, const uint32_t* keys, const
 // smooth top-k loss from the relaxed mask (tk_loss.cu)
 cudaError_t launch_loss(const float* theta, const int32_t* target, float* grad, float* loss, long long rows,
                         int n, double p, double lambda, int q4, double qm1, int vec4, cudaStream_t stream);
+// stable argsort of rows of up to perm_max_n() elements, with the hard operator on request (tk_perm.cu)
+int perm_max_n();
+cudaError_t launch_perm(const float* theta, long long rows, int n, int k, int mode, int32_t* perm, float* sorted,
+                        float* hard, int32_t* status, cudaStream_t stream);
 // hard operators from the permutation (tk_hard.cu)
 cudaError_t launch_hard(const float* theta, const int32_t* perm, float* out, long long rows, int n, int k,
                         int mode, cudaStream_t stream);
@@ -161,8 +165,9 @@ size_t tk_workspace_bytes(int64_t rows, int64_t n, int64_t k, double p, int mode
   return tk::long_workspace_bytes(rows, (int)n);
 }
 
-static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_t k, double p,
-                             double lambda, int mode, float* out, const tk_opts* opts, tk_stream stream) {
+// hard: out receives the hard operator (straight-through); *hard_done: it has, else the caller makes it from perm_out.
+static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_t k, double p, double lambda, int mode,
+                             float* out, const tk_opts* opts, tk_stream stream, bool hard, bool* hard_done) {
   int q4 = 0;
   double qm1 = 0.0;
   tk_status s = check_common(theta, rows, n, k, p, lambda, mode, &q4, &qm1);
@@ -186,6 +191,20 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
   P.what = tk::W_FWD;
   if (opts) { P.perm_out = opts->perm_out; P.state_out = opts->state_out; P.status = opts->status_out; }
   P.vec4 = (n % 4 == 0) && aligned16(theta) && aligned16(out);
+  // A permutation from AUTO: the order comes from the keys-only sort, the relaxed values and the row state from the
+  // threshold form, which needs no order.  One kernel that sorts 64-bit words and solves on them (and another that makes
+  // the hard output) stays faster up to 32 elements only: 699050 x 24, p = 2: 269 us and 270; 262144 x 64: 221 and 118;
+  // 4194 x 4000: 420 and 265.  A hard output needs the row state alone.
+  if (solver == TK_SOLVER_AUTO && P.perm_out && qm1 == 0.0 && n > 32 && n <= tk::perm_max_n()) {
+    tk::Problem F = P;
+    F.perm_out = nullptr;
+    if (hard) { F.out = nullptr; *hard_done = true; }
+    if (!hard || F.state_out) {
+      if (tk::launch_newton(F, (cudaStream_t)stream) != cudaSuccess) return TK_ERR_CUDA;
+    }
+    return tk::launch_perm(theta, rows, (int)n, (int)k, mode, P.perm_out, nullptr, hard ? out : nullptr, P.status,
+                           (cudaStream_t)stream) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  }
   // phi(x) = x with a closed-form block solve, nothing but values asked for: the threshold form needs no
   // order at all (TK_SOLVER_PAV keeps the sort)
   // (very short rows sort faster than they iterate: AUTO keeps the sort up to 8 elements, up to 16 for p = 4/3)
@@ -256,8 +275,9 @@ tk_status tk_fwd_ex(const float* theta, int64_t rows, int64_t n, int64_t k, doub
   if (opts && (opts->flags & ~TK_OPT_STRAIGHT_THROUGH)) return TK_ERR_INVALID_ARG;
   if (st && rows > 0 && opts->perm_out == nullptr) return TK_ERR_INVALID_ARG;
   if (st && opts->solver == TK_SOLVER_THRESHOLD) return TK_ERR_UNSUPPORTED;
-  tk_status s = fwd_relaxed(theta, rows, n, k, p, lambda, mode, out, opts, stream);
-  if (s != TK_OK || !st || rows == 0) return s;
+  bool hard_done = false;
+  tk_status s = fwd_relaxed(theta, rows, n, k, p, lambda, mode, out, opts, stream, st, &hard_done);
+  if (s != TK_OK || !st || rows == 0 || hard_done) return s;
   // the relaxed pass has left the permutation (and the row state); the hard operator replaces its output
   cudaError_t e = tk::launch_hard(theta, opts->perm_out, out, rows, (int)n, (int)k, mode, (cudaStream_t)stream);
   return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
@@ -522,6 +542,12 @@ tk_status tk_argsort(const float* theta, int64_t rows, int64_t n, int mode, int3
   P.sorted_out = sorted_out;
   if (opts) P.status = opts->status_out;
   P.vec4 = (n % 4 == 0) && aligned16(theta);
+  // (139810 x 120: 112 us with 64-bit words through the network, 93 here; 8388 x 500: 57 and 34; 262144 x 64: 82 and 83, with
+  // a longer latency on few rows; 2097 x 8000: 346 and 394)
+  if (n > 64 && n <= 4096) {
+    cudaError_t ep = tk::launch_perm(theta, rows, (int)n, 1, mode, perm_out, sorted_out, nullptr, P.status, (cudaStream_t)stream);
+    return ep == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  }
   if (n > tk::kMaxOnChipN) {
     tk_status s = check_workspace(opts, rows, n);
     if (s != TK_OK) return s;

@@ -455,6 +455,14 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
     P.state_out[row] = st;
   }
 
+  if (P.out == nullptr) {                      // the row state alone was asked for
+    if (P.status) {
+      if (bad) flags |= TK_FLAG_NONFINITE;
+      if (flags) atomicOr(P.status, flags);
+    }
+    return;
+  }
+
   // ---- dual map y = rho(clamp(key - tau)), in the order the keys were read.  phi even: a top singleton
   // is its own minimiser vtop(key) (stationarity rho(key - v) = v), and the sign of theta comes back
   if (!MAG) {

@@ -30,7 +30,7 @@ namespace {
 
 constexpr int kSwMaxWindow = 512;               // 16 ranks per lane of one warp
 
-// One row's window: the ranks [lo, hi), lo even; arrays by rank - lo (s: padded slots by rank).
+// One row's window: the ranks [lo, hi), lo even; arrays by rank - lo (s: rk_slot of the rank).
 struct SwWin {
   const float* s;          // sorted keys of the row
   float* v;                // p = 2: the iterate; at the end the results
@@ -94,7 +94,7 @@ __device__ __forceinline__ int sw_dykstra(const SwWin& Wn, float lam, int it, in
 }
 
 // p = 4/3, phi = x: H pairs per lane, round-robin over GG lanes (pair q = ranks lo + 2q, lo + 2q + 1 of the part)
-template <int H, int GG>
+template <int H, int GG, int G, int W>
 __device__ __forceinline__ int sw_bca(const SwWin& Wn, const Math& M, int it, int sweeps, int l) {
   int lo, hi;
   sw_part(Wn, 2 * GG * H, lo, hi);
@@ -106,9 +106,9 @@ __device__ __forceinline__ int sw_bca(const SwWin& Wn, const Math& M, int it, in
 #pragma unroll
   for (int j = 0; j < H; ++j) {
     const int q = l + j * GG;
-    s_lo[j] = Wn.s[rk_slot(min(lo + 2 * q, hi - 1))];
-    s_hi[j] = Wn.s[rk_slot(min(lo + 2 * q + 1, hi - 1))];
-    s_nx[j] = Wn.s[rk_slot(min(lo + 2 * q + 2, hi - 1))];
+    s_lo[j] = Wn.s[rk_slot<G, W>(min(lo + 2 * q, hi - 1))];
+    s_hi[j] = Wn.s[rk_slot<G, W>(min(lo + 2 * q + 1, hi - 1))];
+    s_nx[j] = Wn.s[rk_slot<G, W>(min(lo + 2 * q + 2, hi - 1))];
     ao[j] = 2 * q < cnt ? al[2 * q] : 0.0f;
     ae[j] = 2 * q + 1 < cnt ? al[2 * q + 1] : 0.0f;
   }
@@ -149,11 +149,11 @@ __device__ __forceinline__ int sw_bca(const SwWin& Wn, const Math& M, int it, in
 }
 
 // All sweeps of a row, and the results of its window into Wn.v.
-template <int GG, bool Q4, bool MAG>
+template <int GG, int G, int W, bool Q4, bool MAG>
 __device__ __forceinline__ void sw_solve(const SwWin& Wn, const Math& M, int sweeps, int l) {
   const int cnt = Wn.hi - Wn.lo;
   for (int j = l; j < cnt; j += GG) {
-    const float sj = Wn.s[rk_slot(Wn.lo + j)];
+    const float sj = Wn.s[rk_slot<G, W>(Wn.lo + j)];
     const bool top = Wn.lo + j < Wn.k;
     if (!Q4) Wn.v[j] = MAG ? (top ? sj / (1.0f + M.lam) : sj) : (top ? sj - M.lam : sj);
     Wn.del[j] = 0.0f;
@@ -161,10 +161,10 @@ __device__ __forceinline__ void sw_solve(const SwWin& Wn, const Math& M, int swe
   __syncwarp();
   int it = 0;
   if (Q4) {
-    if (GG >= 16) it = sw_bca<1, GG>(Wn, M, it, sweeps, l);
-    if (GG >= 4 && it < sweeps) it = sw_bca<2, GG>(Wn, M, it, sweeps, l);
-    if (GG >= 16 && it < sweeps) it = sw_bca<4, GG>(Wn, M, it, sweeps, l);
-    if (it < sweeps) sw_bca<8, GG>(Wn, M, it, sweeps, l);
+    if (GG >= 16) it = sw_bca<1, GG, G, W>(Wn, M, it, sweeps, l);
+    if (GG >= 4 && it < sweeps) it = sw_bca<2, GG, G, W>(Wn, M, it, sweeps, l);
+    if (GG >= 16 && it < sweeps) it = sw_bca<4, GG, G, W>(Wn, M, it, sweeps, l);
+    if (it < sweeps) sw_bca<8, GG, G, W>(Wn, M, it, sweeps, l);
   } else {
     if (GG >= 16) it = sw_dykstra<2, GG, MAG>(Wn, M.lam, it, sweeps, l);
     if (GG >= 4 && it < sweeps) it = sw_dykstra<4, GG, MAG>(Wn, M.lam, it, sweeps, l);
@@ -173,7 +173,7 @@ __device__ __forceinline__ void sw_solve(const SwWin& Wn, const Math& M, int swe
   }
   for (int j = l; j < cnt; j += GG) {
     if (Q4) Wn.v[j] = (Wn.lo + j < Wn.k ? 1.0f : 0.0f) - Wn.del[j] + (j > 0 ? Wn.del[j - 1] : 0.0f);
-    else Wn.v[j] = (Wn.s[rk_slot(Wn.lo + j)] - (MAG ? fmaxf(Wn.v[j], 0.0f) : Wn.v[j])) * M.inv_lam;
+    else Wn.v[j] = (Wn.s[rk_slot<G, W>(Wn.lo + j)] - (MAG ? fmaxf(Wn.v[j], 0.0f) : Wn.v[j])) * M.inv_lam;
   }
   if (l == 0) { Wn.v[cnt] = 0.0f; Wn.v[cnt + 1] = 1.0f; }
 }
@@ -222,44 +222,19 @@ __global__ void __launch_bounds__(RankGeom<G, W>::THREADS, (W == 1 ? 5 : (W >= 1
     r[i] = lig + T * i < n ? key[i] : -INFINITY;
   }
   rank_sort<G, W>(r, tid, sm[team]);
-#pragma unroll
-  for (int i = 0; i < E; ++i) s[lig * (E + 1) + i] = r[i];
-  rk_sync<W>();
+  bool tie = rank_store<G, W>(r, s, n, lig);
 
   // ---- every element's place in the window: 0 .. cnt - 1, cnt below it, cnt + 1 above it
   int at[E];
-  bool tie = P.perm_out != nullptr;
-  {
-    const float top = s[rk_slot(lo)];
-    int st0 = 1;
-    while (2 * st0 <= cnt) st0 <<= 1;
 #pragma unroll
-    for (int i = 0; i < E; ++i) at[i] = 0;
-#pragma unroll 1
-    for (int st = st0; st > 0; st >>= 1) {
-#pragma unroll
-      for (int i = 0; i < E; ++i) {
-        const int q = at[i] + st;
-        if (q <= cnt && s[rk_slot(lo + min(q, cnt) - 1)] > key[i]) at[i] = q;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < E; ++i) {
-      tie |= lig + T * i < n && at[i] < cnt && lo + at[i] + 1 < n && s[rk_slot(lo + at[i] + 1)] == key[i];
-      if (key[i] > top) at[i] = cnt + 1;
-    }
-  }
+  for (int i = 0; i < E; ++i) at[i] = rank_find<G, W>(s, n, key[i]);
   tie = W > 1 ? __syncthreads_or(tie) != 0 : __any_sync(0xffffffffu, tie);
-  if (tie) {                                                      // equal keys: by their ranks in the whole row
+  if (tie) rank_ties<G, W>(at, s, n, lig, rl, tid, reinterpret_cast<int*>(work));
 #pragma unroll
-    for (int i = 0; i < E; ++i) at[i] = rank_find<G, W>(s, n, key[i]);
-    rank_ties<G, W>(at, s, n, lig, rl, tid, reinterpret_cast<int*>(work));
-#pragma unroll
-    for (int i = 0; i < E; ++i) {
-      const int e = lig + T * i;
-      if (P.perm_out && live && e < n) P.perm_out[first + at[i]] = e;
-      at[i] = at[i] < lo ? cnt + 1 : (at[i] < hi ? at[i] - lo : cnt);
-    }
+  for (int i = 0; i < E; ++i) {
+    const int e = lig + T * i;
+    if (P.perm_out && live && e < n) P.perm_out[first + at[i]] = e;
+    at[i] = at[i] < lo ? cnt + 1 : (at[i] < hi ? at[i] - lo : cnt);
   }
 
   // ---- the sweeps: the row's lanes, or the first warp of its warps
@@ -268,7 +243,7 @@ __global__ void __launch_bounds__(RankGeom<G, W>::THREADS, (W == 1 ? 5 : (W >= 1
   if (W == 1 || threadIdx.x < 32) {
     SwWin Wn;
     Wn.s = s; Wn.v = ys; Wn.del = ys + SwGeom<G, W>::VN; Wn.lo = lo; Wn.hi = hi; Wn.k = P.k;
-    sw_solve<W == 1 ? G : 32, Q4, MAG>(Wn, M, P.sweeps > 0 ? P.sweeps : 100, W == 1 ? lig : lane);
+    sw_solve<W == 1 ? G : 32, G, W, Q4, MAG>(Wn, M, P.sweeps > 0 ? P.sweeps : 100, W == 1 ? lig : lane);
   }
   rk_sync<W>();
 

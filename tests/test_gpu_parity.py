@@ -1064,3 +1064,31 @@ def test_sweeps_on_the_ranks_they_reach(n):
                 ref = tko.dykstra(x, k, p, 0.7, mode, sweeps=sweeps)
                 assert rel_err(out.cpu().numpy(), ref).max() <= 1e-5, (n, sweeps, k, mode, want_perm)
             assert np.array_equal(perm.cpu().numpy(), tko.argsort(x, mode)[0]), (n, sweeps, mode)
+
+
+@pytest.mark.parametrize("n", [1, 2, 16, 17, 32, 33, 65, 128, 129, 256, 257, 512, 513, 1024, 1025, 2048, 2049, 4096, 4097, 8191, 8192])
+def test_stable_argsort_at_team_edges(n):
+    """tk_argsort and the straight-through output around every change of the sorting team: few equal keys (listed), long
+    runs of them (walked), signed zeros, infinities, a ragged last row of a warp; bit-exact against the oracle."""
+    from oracle import tko
+    rows = 41 if n <= 128 else 7
+    x = rows_of(n, rows, 9000 + n, 1.0)
+    x[1] = np.round(x[1] * 4) / 4
+    x[2, :] = -1.5
+    if n >= 16:
+        x[3, [2, 5, 11]] = x[3, 7]
+        x[4, ::3] = 0.0
+        x[4, 1::3] = -0.0
+    th = torch.from_numpy(x).cuda()
+    k = max(1, n // 5)
+    for mode in (tk.TK_MASK, tk.TK_TOPK, tk.TK_TOPKMAG):
+        perm = torch.full((rows, n), -1, dtype=torch.int32, device="cuda")
+        srt = torch.empty_like(th)
+        tk.tk_argsort(th, rows, n, mode, perm, srt)
+        perm2, out, state = torch.full_like(perm, -1), torch.empty_like(th), tk.new_state(rows)
+        tk.tk_fwd_ex(th, rows, n, k, 2.0, 0.5, mode, out, perm_out=perm2, state_out=state, flags=tk.TK_OPT_STRAIGHT_THROUGH)
+        torch.cuda.synchronize()
+        rp, rs = tko.argsort(x, mode)
+        assert np.array_equal(perm.cpu().numpy(), rp) and np.array_equal(perm2.cpu().numpy(), rp), (n, mode)
+        assert np.array_equal(srt.cpu().numpy().astype(np.float64), rs), (n, mode)
+        assert np.array_equal(out.cpu().numpy().astype(np.float64), tko.hard(x, k, mode)), (n, mode)
