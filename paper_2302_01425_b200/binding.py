@@ -4,6 +4,10 @@ Every function here has the name and the arguments of its C counterpart in
 include/tk.h; tensors are torch CUDA tensors used purely as device buffers and
 work is enqueued on torch's current stream.  There is no CPU path: loading
 fails loudly when the library has not been built.
+
+A call goes through _tk_bind (csrc/host/tk_bind.cpp: the same checks and the same call in C++, 1 us
+instead of 8); what it does not take -- no library bound yet, or an argument that fails a check --
+it hands back, and the ctypes code below loads the library or raises the error.
 """
 from __future__ import annotations
 
@@ -12,6 +16,11 @@ import os
 from typing import Optional
 
 import torch
+
+try:
+    from . import _tk_bind as _native
+except ImportError:             # not built yet: every call takes the ctypes code
+    _native = None
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libtk.so")
@@ -28,6 +37,9 @@ EXPORTS = ("tk_version", "tk_status_string", "tk_workspace_bytes", "tk_fwd", "tk
            "tk_jvp", "tk_argsort", "tk_fwd_noalloc", "tk_topk_loss",
            "tk_cols_workspace_bytes", "tk_fwd_cols", "tk_vjp_cols", "tk_fwd_w", "tk_vjp_w")
 TK_NOALLOC_MAX_ELEMENTS = 1 << 18
+# the entry points _tk_bind calls, in the order it takes their addresses
+_NATIVE_ENTRIES = ("tk_fwd", "tk_fwd_noalloc", "tk_fwd_ex", "tk_vjp", "tk_jvp", "tk_topk_loss", "tk_fwd_cols",
+                   "tk_vjp_cols", "tk_argsort", "tk_fwd_w", "tk_vjp_w")
 
 
 class TkOpts(ctypes.Structure):
@@ -59,6 +71,8 @@ def use_library(path: str) -> None:
     global _lib, LIB_PATH
     LIB_PATH = path
     _lib = None
+    if _native is not None:
+        _native.bind()
 
 
 def load() -> ctypes.CDLL:
@@ -101,6 +115,8 @@ def load() -> ctypes.CDLL:
     lib.tk_argsort.restype = ci
     lib.tk_argsort.argtypes = [vp, i64, i64, ci, vp, vp, ctypes.POINTER(TkOpts), vp]
     _lib = lib
+    if _native is not None:
+        _native.bind(*(ctypes.cast(getattr(lib, f), vp).value for f in _NATIVE_ENTRIES))
     return lib
 
 
@@ -153,8 +169,10 @@ def tk_workspace_bytes(rows: int, n: int, k: int, p: float, mode: int, solver: i
 
 def tk_fwd(theta: torch.Tensor, rows: int, n: int, k: int, p: float, lam: float, mode: int,
            out: torch.Tensor) -> None:
-    rc = load().tk_fwd(_dev(theta, torch.float32, "theta", rows * n), rows, n, k, p, lam, mode,
-                       _dev(out, torch.float32, "out", rows * n), _stream())
+    rc = _native.fwd(rows, n, k, p, lam, mode, theta, out) if _native else None
+    if rc is None:
+        rc = load().tk_fwd(_dev(theta, torch.float32, "theta", rows * n), rows, n, k, p, lam, mode,
+                           _dev(out, torch.float32, "out", rows * n), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_fwd")
 
@@ -163,47 +181,59 @@ def tk_fwd_noalloc(theta: torch.Tensor, rows: int, n: int, k: int, p: float, lam
                    out: torch.Tensor) -> None:
     """tk_fwd for callers that cannot allocate: long rows use the scratch array built into
     the library (rows * n <= TK_NOALLOC_MAX_ELEMENTS; calls must not overlap on the GPU)."""
-    rc = load().tk_fwd_noalloc(_dev(theta, torch.float32, "theta", rows * n), rows, n, k, p, lam, mode,
-                               _dev(out, torch.float32, "out", rows * n), _stream())
+    rc = _native.fwd_noalloc(rows, n, k, p, lam, mode, theta, out) if _native else None
+    if rc is None:
+        rc = load().tk_fwd_noalloc(_dev(theta, torch.float32, "theta", rows * n), rows, n, k, p, lam, mode,
+                                   _dev(out, torch.float32, "out", rows * n), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_fwd_noalloc")
 
 
 def tk_fwd_ex(theta, rows, n, k, p, lam, mode, out, *, solver=TK_SOLVER_AUTO, sweeps=0,
               perm_out=None, state_out=None, workspace=None, status_out=None, flags=0, tol=0.0) -> None:
-    o = _opts(solver, sweeps, perm_out, state_out, workspace, status_out, flags, rows=rows, n=n, tol=tol)
-    rc = load().tk_fwd_ex(_dev(theta, torch.float32, "theta", rows * n), rows, n, k, p, lam, mode,
-                          _dev(out, torch.float32, "out", rows * n), ctypes.byref(o), _stream())
+    rc = _native.fwd_ex(rows, n, k, p, lam, mode, theta, out, solver, sweeps, perm_out,
+                        state_out, workspace, status_out, flags, tol) if _native else None
+    if rc is None:
+        o = _opts(solver, sweeps, perm_out, state_out, workspace, status_out, flags, rows=rows, n=n, tol=tol)
+        rc = load().tk_fwd_ex(_dev(theta, torch.float32, "theta", rows * n), rows, n, k, p, lam, mode,
+                              _dev(out, torch.float32, "out", rows * n), ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_fwd_ex")
 
 
 def tk_vjp(theta, grad_out, rows, n, k, p, lam, mode, grad_theta, *, state=None, workspace=None,
            status_out=None) -> None:
-    o = _opts(state=state, workspace=workspace, status_out=status_out, rows=rows, n=n)
-    rc = load().tk_vjp(_dev(theta, torch.float32, "theta", rows * n), _dev(grad_out, torch.float32, "grad_out", rows * n),
-                       rows, n, k, p, lam, mode, _dev(grad_theta, torch.float32, "grad_theta", rows * n),
-                       ctypes.byref(o), _stream())
+    rc = _native.vjp(rows, n, k, p, lam, mode, theta, grad_out, grad_theta, state, workspace, status_out) if _native else None
+    if rc is None:
+        o = _opts(state=state, workspace=workspace, status_out=status_out, rows=rows, n=n)
+        rc = load().tk_vjp(_dev(theta, torch.float32, "theta", rows * n), _dev(grad_out, torch.float32, "grad_out", rows * n),
+                           rows, n, k, p, lam, mode, _dev(grad_theta, torch.float32, "grad_theta", rows * n),
+                           ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_vjp")
 
 
 def tk_jvp(theta, tangent, rows, n, k, p, lam, mode, out_tangent, *, state, workspace=None,
            status_out=None) -> None:
-    o = _opts(state=state, workspace=workspace, status_out=status_out, rows=rows, n=n)
-    rc = load().tk_jvp(_dev(theta, torch.float32, "theta", rows * n), _dev(tangent, torch.float32, "tangent", rows * n),
-                       rows, n, k, p, lam, mode, _dev(out_tangent, torch.float32, "out_tangent", rows * n),
-                       ctypes.byref(o), _stream())
+    rc = _native.jvp(rows, n, k, p, lam, mode, theta, tangent, out_tangent, state, workspace, status_out) if _native else None
+    if rc is None:
+        o = _opts(state=state, workspace=workspace, status_out=status_out, rows=rows, n=n)
+        rc = load().tk_jvp(_dev(theta, torch.float32, "theta", rows * n), _dev(tangent, torch.float32, "tangent", rows * n),
+                           rows, n, k, p, lam, mode, _dev(out_tangent, torch.float32, "out_tangent", rows * n),
+                           ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_jvp")
 
 
 def tk_topk_loss(theta, target, rows, n, k, p, lam, loss, grad, *, solver=TK_SOLVER_AUTO, sweeps=0,
                  state_out=None, workspace=None, status_out=None) -> None:
-    o = _opts(solver, sweeps, None, state_out, workspace, status_out, rows=rows, n=n)
-    rc = load().tk_topk_loss(_dev(theta, torch.float32, "theta", rows * n), _dev(target, torch.int32, "target", rows),
-                             rows, n, k, p, lam, _dev(loss, torch.float32, "loss", rows),
-                             _dev(grad, torch.float32, "grad", rows * n), ctypes.byref(o), _stream())
+    rc = _native.topk_loss(rows, n, k, p, lam, theta, target, loss, grad, solver, sweeps, state_out,
+                           workspace, status_out) if _native else None
+    if rc is None:
+        o = _opts(solver, sweeps, None, state_out, workspace, status_out, rows=rows, n=n)
+        rc = load().tk_topk_loss(_dev(theta, torch.float32, "theta", rows * n), _dev(target, torch.int32, "target", rows),
+                                 rows, n, k, p, lam, _dev(loss, torch.float32, "loss", rows),
+                                 _dev(grad, torch.float32, "grad", rows * n), ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_topk_loss")
 
@@ -214,52 +244,64 @@ def tk_cols_workspace_bytes(n: int, cols: int) -> int:
 
 def tk_fwd_cols(theta, n, cols, ld, k, p, lam, mode, out, *, workspace, solver=TK_SOLVER_AUTO, sweeps=0,
                 perm_out=None, state_out=None, status_out=None, flags=0) -> None:
-    o = _opts(solver, sweeps, perm_out, state_out, workspace, status_out, flags, rows=cols, n=n)
-    span = (n - 1) * ld + cols if n > 0 else 0          # last element touched of an [n, cols] matrix with leading dimension ld
-    rc = load().tk_fwd_cols(_dev(theta, torch.float32, "theta", span), n, cols, ld, k, p, lam, mode,
-                            _dev(out, torch.float32, "out", span), ctypes.byref(o), _stream())
+    rc = _native.fwd_cols(n, cols, ld, k, p, lam, mode, theta, out, solver, sweeps, perm_out, state_out,
+                          workspace, status_out, flags) if _native else None
+    if rc is None:
+        o = _opts(solver, sweeps, perm_out, state_out, workspace, status_out, flags, rows=cols, n=n)
+        span = (n - 1) * ld + cols if n > 0 else 0          # last element touched of an [n, cols] matrix with leading dimension ld
+        rc = load().tk_fwd_cols(_dev(theta, torch.float32, "theta", span), n, cols, ld, k, p, lam, mode,
+                                _dev(out, torch.float32, "out", span), ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_fwd_cols")
 
 
 def tk_vjp_cols(theta, grad_out, n, cols, ld, k, p, lam, mode, grad_theta, *, workspace, state=None,
                 status_out=None) -> None:
-    o = _opts(state=state, workspace=workspace, status_out=status_out, rows=cols, n=n)
-    span = (n - 1) * ld + cols if n > 0 else 0
-    rc = load().tk_vjp_cols(_dev(theta, torch.float32, "theta", span), _dev(grad_out, torch.float32, "grad_out", span),
-                            n, cols, ld, k, p, lam, mode, _dev(grad_theta, torch.float32, "grad_theta", span),
-                            ctypes.byref(o), _stream())
+    rc = _native.vjp_cols(n, cols, ld, k, p, lam, mode, theta, grad_out, grad_theta, state, workspace,
+                          status_out) if _native else None
+    if rc is None:
+        o = _opts(state=state, workspace=workspace, status_out=status_out, rows=cols, n=n)
+        span = (n - 1) * ld + cols if n > 0 else 0
+        rc = load().tk_vjp_cols(_dev(theta, torch.float32, "theta", span), _dev(grad_out, torch.float32, "grad_out", span),
+                                n, cols, ld, k, p, lam, mode, _dev(grad_theta, torch.float32, "grad_theta", span),
+                                ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_vjp_cols")
 
 
 def tk_argsort(theta, rows, n, mode, perm_out, sorted_out=None, *, workspace=None,
                status_out=None) -> None:
-    o = _opts(workspace=workspace, status_out=status_out)
-    rc = load().tk_argsort(_dev(theta, torch.float32, "theta", rows * n), rows, n, mode,
-                           _dev(perm_out, torch.int32, "perm_out", rows * n),
-                           _dev(sorted_out, torch.float32, "sorted_out", rows * n), ctypes.byref(o), _stream())
+    rc = _native.argsort(rows, n, mode, theta, perm_out, sorted_out, workspace, status_out) if _native else None
+    if rc is None:
+        o = _opts(workspace=workspace, status_out=status_out)
+        rc = load().tk_argsort(_dev(theta, torch.float32, "theta", rows * n), rows, n, mode,
+                               _dev(perm_out, torch.int32, "perm_out", rows * n),
+                               _dev(sorted_out, torch.float32, "sorted_out", rows * n), ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_argsort")
 
 
 def tk_fwd_w(theta, w, rows, n, p, lam, out, *, status_out=None) -> None:
     """w: [n] (shared by every row) or [rows, n], every row non-increasing."""
-    w_rows = 1 if w.numel() == n and rows != 1 else (rows if w.numel() >= rows * n else 1)
-    o = _opts(status_out=status_out)
-    rc = load().tk_fwd_w(_dev(theta, torch.float32, "theta", rows * n), _dev(w, torch.float32, "w", w_rows * n),
-                         rows, n, w_rows, p, lam, _dev(out, torch.float32, "out", rows * n), ctypes.byref(o), _stream())
+    rc = _native.fwd_w(rows, n, p, lam, theta, w, out, status_out) if _native else None
+    if rc is None:
+        w_rows = 1 if w.numel() == n and rows != 1 else (rows if w.numel() >= rows * n else 1)
+        o = _opts(status_out=status_out)
+        rc = load().tk_fwd_w(_dev(theta, torch.float32, "theta", rows * n), _dev(w, torch.float32, "w", w_rows * n),
+                             rows, n, w_rows, p, lam, _dev(out, torch.float32, "out", rows * n), ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_fwd_w")
 
 
 def tk_vjp_w(theta, w, grad_out, rows, n, p, lam, grad_theta, *, grad_w=None, status_out=None) -> None:
     """grad_w (optional): [rows, n], the cotangent pulled back to w (per row, in w's order)."""
-    w_rows = 1 if w.numel() == n and rows != 1 else (rows if w.numel() >= rows * n else 1)
-    o = _opts(status_out=status_out)
-    rc = load().tk_vjp_w(_dev(theta, torch.float32, "theta", rows * n), _dev(w, torch.float32, "w", w_rows * n),
-                         _dev(grad_out, torch.float32, "grad_out", rows * n), rows, n, w_rows, p, lam,
-                         _dev(grad_theta, torch.float32, "grad_theta", rows * n),
-                         _dev(grad_w, torch.float32, "grad_w", rows * n), ctypes.byref(o), _stream())
+    rc = _native.vjp_w(rows, n, p, lam, theta, w, grad_out, grad_theta, grad_w, status_out) if _native else None
+    if rc is None:
+        w_rows = 1 if w.numel() == n and rows != 1 else (rows if w.numel() >= rows * n else 1)
+        o = _opts(status_out=status_out)
+        rc = load().tk_vjp_w(_dev(theta, torch.float32, "theta", rows * n), _dev(w, torch.float32, "w", w_rows * n),
+                             _dev(grad_out, torch.float32, "grad_out", rows * n), rows, n, w_rows, p, lam,
+                             _dev(grad_theta, torch.float32, "grad_theta", rows * n),
+                             _dev(grad_w, torch.float32, "grad_w", rows * n), ctypes.byref(o), _stream())
     if rc != TK_OK:
         raise TkError(rc, "tk_vjp_w")

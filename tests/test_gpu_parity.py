@@ -1092,3 +1092,49 @@ def test_stable_argsort_at_team_edges(n):
         assert np.array_equal(perm.cpu().numpy(), rp) and np.array_equal(perm2.cpu().numpy(), rp), (n, mode)
         assert np.array_equal(srt.cpu().numpy().astype(np.float64), rs), (n, mode)
         assert np.array_equal(out.cpu().numpy().astype(np.float64), tko.hard(x, k, mode)), (n, mode)
+
+
+def test_native_and_ctypes_marshalling_agree(monkeypatch):
+    """Every call through _tk_bind gives the bits of the same call through ctypes; what _tk_bind does not take (short,
+    strided or wrongly typed buffers) raises the ctypes code's error."""
+    from paper_2302_01425_b200 import binding as b
+    assert b._native is not None, "csrc/host/tk_bind.cpp has not been built"
+    rows, n, k, lam = 33, 96, 7, 0.7
+    th = torch.from_numpy(rows_of(n, rows, 31, 1.0)).cuda()
+    g = torch.from_numpy(rows_of(n, rows, 32, 1.0)).cuda()
+    w = torch.arange(n, 0, -1, device="cuda", dtype=torch.float32)
+    target = torch.arange(rows, device="cuda", dtype=torch.int32)
+
+    def everything():
+        got = []
+        def f32(*shape):
+            got.append(torch.full(shape, -3.0, device="cuda"))
+            return got[-1]
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        state, perm = tk.new_state(rows), torch.zeros(rows, n, dtype=torch.int32, device="cuda")
+        ws = torch.empty(tk.tk_cols_workspace_bytes(rows, n), dtype=torch.uint8, device="cuda")
+        tk.tk_fwd(th, rows, n, k, 2.0, lam, tk.TK_MASK, f32(rows, n))
+        tk.tk_fwd_noalloc(th, rows, n, k, P43, lam, tk.TK_TOPK, f32(rows, n))
+        tk.tk_fwd_ex(th, rows, n, k, 2, 1, tk.TK_TOPKMAG, f32(rows, n), state_out=state, perm_out=perm, status_out=status)
+        tk.tk_vjp(th, g, rows, n, k, 2, 1, tk.TK_TOPKMAG, f32(rows, n), state=state)
+        tk.tk_jvp(th, g, rows, n, k, 2, 1, tk.TK_TOPKMAG, f32(rows, n), state=state)
+        tk.tk_topk_loss(th, target, rows, n, k, P43, lam, f32(rows), f32(rows, n))
+        tk.tk_fwd_cols(th, rows, n, n, 5, 2.0, lam, tk.TK_MASK, f32(rows, n), workspace=ws, state_out=(st2 := tk.new_state(n)))
+        tk.tk_vjp_cols(None, g, rows, n, n, 5, 2.0, lam, tk.TK_MASK, f32(rows, n), workspace=ws, state=st2)
+        tk.tk_argsort(th, rows, n, tk.TK_MASK, perm2 := torch.zeros_like(perm), f32(rows, n))
+        tk.tk_fwd_w(th, w, rows, n, 2.0, lam, f32(rows, n))
+        tk.tk_vjp_w(th, w, g, rows, n, P43, lam, f32(rows, n), grad_w=f32(rows, n))
+        torch.cuda.synchronize()
+        return [t.cpu() for t in got + [perm, perm2, status]]
+
+    native = everything()
+    with monkeypatch.context() as m:
+        m.setattr(b, "_native", None)
+        plain = everything()
+    assert all(torch.equal(x, y) for x, y in zip(native, plain)) and len(native) == len(plain)
+    out = torch.empty_like(th)
+    for bad in (th[:, :-1], th.double(), th.cpu(), th.flatten()[:-1]):
+        with pytest.raises(ValueError, match="theta"):
+            tk.tk_fwd(bad, rows, n, k, 2.0, lam, tk.TK_MASK, out)
+    with pytest.raises(tk.TkError):
+        tk.tk_fwd(th, rows, n, n + 1, 2.0, lam, tk.TK_MASK, out)
