@@ -11,7 +11,7 @@
 // point tightens:
 //   - a step that leaves the bracket is replaced by a step of doubling length towards the root,
 //     then by bisection (of the ordered integer keys when the bracket spans many binades), and
-//     after six Newton steps in a row one such step is forced: the loop ends;
+//     after six Newton steps in a row such steps are forced, larger each time: the loop ends;
 //   - the root is accepted when a point reproduces the set of the pass before it and already
 //     solves it to rounding, or when cm |du| is rounding-sized (F has slope >= 1/lambda until
 //     it reaches an integer, so the root is then within that distance).
@@ -92,7 +92,8 @@ struct NtRow {
   float lo_o, hi_o;          // bracket of the offset: F > 0 at lo_o, F <= 0 at hi_o
   float lo_a, hi_a;          // the same bracket as absolute values of tau
   int prev_ct, prev_cm;      // classes of the pass before
-  int gallop, nnewt;
+  int gallop;
+  int nnewt;                 // Newton steps in a row (low four bits), forced steps so far (above)
   bool edge_tried;
   int a0, b0;
   bool done, noblock, repiv;
@@ -110,13 +111,18 @@ static __device__ __noinline__ NtRow nt_step_slow(NtRow S, int ct, int cm, int m
     cand = S.off + du;
     // every inside key would have to reach the cap: aim just past it, so that they read as capped
     if (nudge) cand -= 0.5f * tol;
-    ok = cand > S.lo_o && cand < S.hi_o && S.nnewt < 6;
+    ok = cand > S.lo_o && cand < S.hi_o && (S.nnewt & 15) < 6;
     nxt = cand;
   }
   if (ok) {
     S.gallop = 0; S.nnewt++;
   } else {
-    S.nnewt = 0;
+    // Six Newton steps without an end: far from the root (heavy tails) each may advance by a few widths only.  The next
+    // steps are forced, 1, 8 and 64 widths, then halvings of the bracket, one after every three Newton steps.
+    const int forced = S.nnewt >> 4;
+    const bool stalled = (S.nnewt & 15) >= 6;
+    S.nnewt = stalled ? ((forced + 1) << 4 | 3) : forced << 4;
+    if (stalled) S.gallop = forced < 3 ? 3 * forced : 8;
     const float width = S.hi_o - S.lo_o;
     if (have && !S.edge_tried && (cand <= S.lo_o || cand >= S.hi_o)) {
       // The piece's root lies at the end of the bracket or a hair beyond it: the true root is
@@ -220,7 +226,7 @@ __device__ __forceinline__ void nt_step(NtRow& S, int ct, int cm, float s1, floa
   // the common case: the piece's solution lies inside the bracket and near the pivot
   const float cand = S.off + du;
   const bool nudge = m == cm;                  // every inside key would have to reach the cap
-  if (have && !nudge && cand > S.lo_o && cand < S.hi_o && S.nnewt < 6 && fabsf(cand) <= 8.0f * wid &&
+  if (have && !nudge && cand > S.lo_o && cand < S.hi_o && (S.nnewt & 15) < 6 && fabsf(cand) <= 8.0f * wid &&
       !(MAG && S.piv + cand < 0.5f * S.piv)) {
     S.gallop = 0; S.nnewt++; S.off = cand;
     return;

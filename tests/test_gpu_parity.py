@@ -1138,3 +1138,21 @@ def test_native_and_ctypes_marshalling_agree(monkeypatch):
             tk.tk_fwd(bad, rows, n, k, 2.0, lam, tk.TK_MASK, out)
     with pytest.raises(tk.TkError):
         tk.tk_fwd(th, rows, n, n + 1, 2.0, lam, tk.TK_MASK, out)
+
+
+@pytest.mark.parametrize("n,k", [(900, 9), (4096, 40), (300000, 3000)])
+def test_heavy_tailed_rows_converge(n, k):
+    """Ratios of normals: the moment start lands hundreds of widths from the root, where every Newton step advances by a few
+    widths (the 300000-element row, p = 4/3, stopped at the 200-pass cap before the forced steps grew)."""
+    from oracle import tko
+    from parity import rel_err, TOL
+    x = rows_of(n, 1, 11000 + n % 997, 1.0)
+    x = (x / np.maximum(np.abs(rows_of(n, 1, 11, 1.0)), 1e-3)).astype(np.float32)
+    th = torch.from_numpy(x).cuda()
+    for mode, p in ((tk.TK_MASK, P43), (tk.TK_TOPK, 2.0), (tk.TK_TOPKMAG, P43)):
+        ws = torch.empty(max(1, tk.tk_workspace_bytes(1, n, k, p, mode)), dtype=torch.uint8, device="cuda")
+        out, status = torch.empty_like(th), torch.zeros(1, dtype=torch.int32, device="cuda")
+        tk.tk_fwd_ex(th, 1, n, k, p, 0.05, mode, out, workspace=ws, status_out=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0, (mode, p)
+        assert rel_err(out.cpu().numpy(), tko.fwd(x, k, p, 0.05, mode)).max() <= TOL, (mode, p)
