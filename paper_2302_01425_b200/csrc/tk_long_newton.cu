@@ -8,8 +8,11 @@
 // power sums, the blocks meet at a grid barrier (cooperative launch: all blocks are resident),
 // and every block then adds the per-block partial sums in the same order and takes the same
 // step.  Two partial-sum buffers alternate, so one grid barrier per pass is enough.  No sort, no
-// histogram: 5 to 10 passes of 2 to 3 microseconds instead of four radix passes over (key, index)
-// pairs.
+// histogram: 5 to 10 passes instead of four radix passes over (key, index) pairs.
+//
+// A pass costs 4 to 5 us, two of them the grid barrier; the classification (two compares and predicated adds per key) and
+// the sums (counts by one warp reduction each, slots as 16-byte words) 2 us on 4194304 elements: 43.1 -> 38.2 us, 1143022
+// elements at p = 4/3 40.1 -> 34.8, against selects and five shuffles per sum and value.
 #include <cooperative_groups.h>
 
 #include "tk_newton_core.cuh"
@@ -25,49 +28,54 @@ constexpr int kLnSlots = 8;                 // words per block and buffer: three
 
 struct LnAcc {
   float v0, v1, v2;
-  uint32_t cnt, cnt2;
+  uint32_t cnt, cnt2;                       // inside, capped
 };
+
+// Sum over the block; every thread returns the same.
+__device__ __forceinline__ LnAcc ln_block_sum(LnAcc x, float* sh) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    x.v0 += __shfl_xor_sync(0xffffffffu, x.v0, o);
+    x.v1 += __shfl_xor_sync(0xffffffffu, x.v1, o);
+    x.v2 += __shfl_xor_sync(0xffffffffu, x.v2, o);
+  }
+  x.cnt = __reduce_add_sync(0xffffffffu, x.cnt);
+  x.cnt2 = __reduce_add_sync(0xffffffffu, x.cnt2);
+  __syncthreads();                             // sh may still be read from the sum before
+  if (lane == 0) {
+    sh[warp * 5] = x.v0; sh[warp * 5 + 1] = x.v1; sh[warp * 5 + 2] = x.v2;
+    sh[warp * 5 + 3] = __uint_as_float(x.cnt); sh[warp * 5 + 4] = __uint_as_float(x.cnt2);
+  }
+  __syncthreads();
+  LnAcc r{0.f, 0.f, 0.f, 0u, 0u};
+#pragma unroll
+  for (int w = 0; w < kLnThreads / 32; ++w) {
+    r.v0 += sh[w * 5]; r.v1 += sh[w * 5 + 1]; r.v2 += sh[w * 5 + 2];
+    r.cnt += __float_as_uint(sh[w * 5 + 3]); r.cnt2 += __float_as_uint(sh[w * 5 + 4]);
+  }
+  return r;
+}
 
 // Sum over the whole grid: block tree, one slot per block in `buf`, grid barrier, then every block adds
 // all slots in the same order (thread t takes slots t, t + 256, ...; then the same block tree).
 __device__ __forceinline__ LnAcc ln_grid_sum(LnAcc a, float* buf, float* sh, cg::grid_group& grid) {
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  auto block_sum = [&](LnAcc x) -> LnAcc {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      x.v0 += __shfl_xor_sync(0xffffffffu, x.v0, o);
-      x.v1 += __shfl_xor_sync(0xffffffffu, x.v1, o);
-      x.v2 += __shfl_xor_sync(0xffffffffu, x.v2, o);
-      x.cnt += __shfl_xor_sync(0xffffffffu, x.cnt, o);
-      x.cnt2 += __shfl_xor_sync(0xffffffffu, x.cnt2, o);
-    }
-    __syncthreads();                           // sh may still be read from the sum before
-    if (lane == 0) {
-      sh[warp * 5] = x.v0; sh[warp * 5 + 1] = x.v1; sh[warp * 5 + 2] = x.v2;
-      sh[warp * 5 + 3] = __uint_as_float(x.cnt); sh[warp * 5 + 4] = __uint_as_float(x.cnt2);
-    }
-    __syncthreads();
-    LnAcc r{0.f, 0.f, 0.f, 0u, 0u};
-#pragma unroll
-    for (int w = 0; w < kLnThreads / 32; ++w) {
-      r.v0 += sh[w * 5]; r.v1 += sh[w * 5 + 1]; r.v2 += sh[w * 5 + 2];
-      r.cnt += __float_as_uint(sh[w * 5 + 3]); r.cnt2 += __float_as_uint(sh[w * 5 + 4]);
-    }
-    return r;
-  };
-  const LnAcc b = block_sum(a);
+  const int t = threadIdx.x;
+  const LnAcc b = ln_block_sum(a, sh);
   if (t == 0) {
-    float* s = buf + (size_t)blockIdx.x * kLnSlots;
-    s[0] = b.v0; s[1] = b.v1; s[2] = b.v2; s[3] = __uint_as_float(b.cnt); s[4] = __uint_as_float(b.cnt2);
+    float4* s = reinterpret_cast<float4*>(buf + (size_t)blockIdx.x * kLnSlots);
+    s[0] = make_float4(b.v0, b.v1, b.v2, __uint_as_float(b.cnt));
+    s[1] = make_float4(__uint_as_float(b.cnt2), 0.0f, 0.0f, 0.0f);
   }
   grid.sync();
   LnAcc p{0.f, 0.f, 0.f, 0u, 0u};
   for (int i = t; i < (int)gridDim.x; i += kLnThreads) {
-    const float* s = buf + (size_t)i * kLnSlots;
-    p.v0 += __ldcg(s); p.v1 += __ldcg(s + 1); p.v2 += __ldcg(s + 2);
-    p.cnt += __float_as_uint(__ldcg(s + 3)); p.cnt2 += __float_as_uint(__ldcg(s + 4));
+    const float4* s = reinterpret_cast<const float4*>(buf + (size_t)i * kLnSlots);
+    const float4 u = __ldcg(s), w = __ldcg(s + 1);
+    p.v0 += u.x; p.v1 += u.y; p.v2 += u.z;
+    p.cnt += __float_as_uint(u.w); p.cnt2 += __float_as_uint(w.x);
   }
-  return block_sum(p);
+  return ln_block_sum(p, sh);
 }
 
 // smallest value over the grid (same scheme; buf slot 0)
@@ -99,6 +107,7 @@ __device__ __forceinline__ void ln_for_each(const float* x_row, int n, int vec4,
   const long long first = (long long)blockIdx.x * kLnThreads + threadIdx.x;
   if (vec4) {
     const float4* x4 = reinterpret_cast<const float4*>(x_row);
+#pragma unroll 4
     for (long long v = first; 4 * v < n; v += stride) {
       if (!TK_IN_BOUNDS(4 * v, 4, n, status)) continue;
       const float4 q = __ldg(x4 + v);
@@ -129,7 +138,9 @@ __global__ void __launch_bounds__(kLnThreads) tk_long_newton_kernel(const Proble
     NtRow S;
     nt_row_init(S, k);
     float wid = lam;
-    // ---- start: moments of the keys (about the first key; phi even: about 0, and the keys above 0 counted)
+    // ---- start: moments of the keys (about the first key; phi even: about 0, and the keys above 0 counted).  Of the
+    // whole row: a sample of 4096 elements, which saves this pass, costs p = 4/3 more passes than it saves (1143022
+    // elements: 40 -> 61 us)
     const float x0 = MAG ? 0.0f : __ldg(x_row);
     LnAcc a{0.f, 0.f, 0.f, 0u, 0u};
     bool bad = false;
@@ -175,14 +186,11 @@ __global__ void __launch_bounds__(kLnThreads) tk_long_newton_kernel(const Proble
       const float tol = kTolRel * (MAG ? fminf(wid, fmaxf(S.piv + S.off, 0.0f)) : wid);
       const float piv = S.piv, off = S.off;
       LnAcc c{0.f, 0.f, 0.f, 0u, 0u};
+      float ct = 0.f, cm = 0.f;                // (exact: a thread's share is below 2^24 keys)
       ln_for_each<MAG>(x_row, n, P.vec4, P.status, [&](float x, long long) {
-        const float t = ((MAG ? fabsf(x) : x) - piv) - off;
-        const bool top = t >= wid, mid = t > 0.0f && !top;
-        c.cnt2 += top; c.cnt += mid;
-        const float tm = mid ? t : 0.0f;
-        c.v0 += tm;
-        if (Q4) { const float t2 = tm * tm; c.v1 += t2; c.v2 = fmaf(t2, tm, c.v2); }
+        nt_classify<Q4>(((MAG ? fabsf(x) : x) - piv) - off, wid, ct, cm, c.v0, c.v1, c.v2);
       });
+      c.cnt2 = (uint32_t)ct; c.cnt = (uint32_t)cm;
       c = ln_grid_sum(c, buf[phase & 1], sh, grid);
       ++phase;
       nt_step<Q4, MAG>(S, (int)c.cnt2, (int)c.cnt, c.v0, c.v1, c.v2, k, lam, lam3, wid, tol);

@@ -1156,3 +1156,37 @@ def test_heavy_tailed_rows_converge(n, k):
         torch.cuda.synchronize()
         assert int(status.item()) == 0, (mode, p)
         assert rel_err(out.cpu().numpy(), tko.fwd(x, k, p, 0.05, mode)).max() <= TOL, (mode, p)
+
+
+@pytest.mark.parametrize("n,kind", [(32769, "normal"), (65537, "sorted"), (606208, "normal"), (606211, "sorted"), (300000, "cauchy"),
+                                    (1000003, "grid"), (250000, "two_scales"), (8486913, "normal")])
+def test_long_rows_over_the_grid(n, kind):
+    """The long-row forward pass and VJP: rows that fill their tiles and ragged ones, sorted rows (the pooled keys in one
+    tile), heavy tails, repeated values, two scales; the same bits from call to call."""
+    from oracle import tko
+    from parity import rel_err, TOL
+    x = rows_of(n, 1, 11000 + n % 997, 1.0)
+    if kind == "sorted":
+        x = np.ascontiguousarray(-np.sort(-np.abs(x), axis=1))
+    elif kind == "cauchy":
+        x = (x / np.maximum(np.abs(rows_of(n, 1, 11, 1.0)), 1e-3)).astype(np.float32)
+    elif kind == "grid":
+        x = (np.round(x * 64) / 64).astype(np.float32)
+    elif kind == "two_scales":
+        x[:, ::2] *= 1e-3
+    g = rows_of(n, 1, 12000 + n % 997, 1.0)
+    th, gt = torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda()
+    cases = ((tk.TK_TOPKMAG, 2.0, 1e-3, n // 10), (tk.TK_MASK, P43, 0.05, n // 100), (tk.TK_TOPK, 2.0, 1e-3, n // 3), (tk.TK_TOPKMAG, P43, 1e-2, 17))
+    for mode, p, lam, k in cases[:1] if n > 4000000 else cases:
+        ws = torch.empty(tk.tk_workspace_bytes(1, n, k, p, mode), dtype=torch.uint8, device="cuda")
+        out, grad, again, state = torch.empty_like(th), torch.empty_like(th), torch.empty_like(th), tk.new_state(1)
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        tk.tk_fwd_ex(th, 1, n, k, p, lam, mode, out, state_out=state, workspace=ws, status_out=status)
+        tk.tk_vjp(th, gt, 1, n, k, p, lam, mode, grad, state=state, workspace=ws)
+        tk.tk_fwd_ex(th, 1, n, k, p, lam, mode, again, workspace=ws)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0 and torch.equal(out, again), (kind, mode, p)
+        assert rel_err(out.cpu().numpy(), tko.fwd(x, k, p, lam, mode)).max() <= TOL, (kind, mode, p)
+        # (the gradient jumps where an element enters the pooled block: elements within 1e-5 of its edge are left out)
+        o, e = out.cpu().numpy().astype(np.float64), rel_err(grad.cpu().numpy(), tko.vjp(x, g, k, p, lam, mode))
+        assert (e > TOL).sum() <= 2, (kind, mode, p, int((e > TOL).sum()), e.max())
