@@ -116,10 +116,12 @@ struct ColMatrix {
   __device__ __forceinline__ ColMatrix(const float* m, long long ld, long long col0, int c, const ColRows<Off>& R, long long cols, int32_t* st)
       : base(reinterpret_cast<const char*>(m + col0)), first((Off)c * 4), step((Off)R.S * (Off)ld * 4),
         lane_off((Off)c * 4 + (Off)R.sl * (Off)ld * 4), extent(((R.n - 1) * ld + cols - col0) * 4), status(st) {}
-  template <bool FAST>
-  __device__ __forceinline__ float load(int i, const ColRows<Off>& R) const {     // past the column's end: its first row
+  // past the column's end: its first row.  AGAIN: read before, the read-only path may be taken
+  template <bool FAST, bool AGAIN = false>
+  __device__ __forceinline__ float load(int i, const ColRows<Off>& R) const {
     const Off o = FAST || R.in(i) ? lane_off + (Off)i * step : first;
-    return TK_IN_BOUNDS(o, 4, extent, status) ? __ldg(reinterpret_cast<const float*>(base + o)) : 0.0f;
+    const float* at = reinterpret_cast<const float*>(base + o);
+    return TK_IN_BOUNDS(o, 4, extent, status) ? (AGAIN ? __ldg(at) : *at) : 0.0f;
   }
   template <bool FAST>
   __device__ __forceinline__ void store(int i, const ColRows<Off>& R, bool col_ok, float v) const {
@@ -162,6 +164,7 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
   constexpr float kTolRel = Q4 ? 1e-7f : 3e-7f;
   int phase = 0;
 
+  overlap_wait();
   float d[E];
   col_each<E>(R, [&](int i, auto fast) { d[i] = X.template load<decltype(fast)::value>(i, R); });
   if (A.copy) {
@@ -257,7 +260,7 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const int i = 4 * g + j;
-              const float xv = Xp.template load<false>(i, Rp);
+              const float xv = Xp.template load<false, true>(i, Rp);
               d[i] = Rp.in(i) ? (MAG ? fabsf(xv) : xv) - T.piv : -INFINITY;
             }
             asm volatile("" ::: "memory");     // loads of the next group stay behind: the registers are full here
@@ -288,7 +291,7 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int i = 4 * g + j;
-            const float xv = Xp.template load<false>(i, Rp);
+            const float xv = Xp.template load<false, true>(i, Rp);
             if (Rp.in(i) && d[i] - T.off >= wid) cmin = fminf(cmin, MAG ? fabsf(xv) : xv);
           }
           asm volatile("" ::: "memory");
@@ -323,7 +326,7 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
     col_each<E>(Ro, [&](int i, auto fast) {
       const float a = __saturatef(fmaf(d[i], inv_lam, shift));
       float y = Q4 ? a * a * a : a;
-      if (times_x) y *= Xo.template load<decltype(fast)::value>(i, Ro);
+      if (times_x) y *= Xo.template load<decltype(fast)::value, true>(i, Ro);
       O.template store<decltype(fast)::value>(i, Ro, col_ok, y);
       if (times_x && (i & 3) == 3) asm volatile("" ::: "memory");
     });
@@ -332,7 +335,7 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
     M.q4 = Q4; M.mag = true; M.gen = false;
     const float off = T.off;
     col_each<E>(Ro, [&](int i, auto fast) {
-      const float xv = Xo.template load<decltype(fast)::value>(i, Ro);
+      const float xv = Xo.template load<decltype(fast)::value, true>(i, Ro);
       const float t = d[i] - off;
       float v = 0.0f;
       if (t >= wid) v = M.vtop(fabsf(xv));
@@ -361,6 +364,7 @@ __global__ void __maxnreg__(E <= 16 ? (MODE == TK_MASK ? 56 : 64) : 112) tk_cols
   const ColRows<Off> R(n);
   const ColMatrix<Off> X(A.theta, A.ld_theta, col0, c, R, cols, P.status);
   const ColMatrix<Off> GM(A.gout, A.ld_gout, col0, c, R, cols, P.status);
+  overlap_wait();
   float x[E], g[E];
   col_each<E>(R, [&](int i, auto fast) {
     x[i] = X.template load<decltype(fast)::value>(i, R);
@@ -444,31 +448,33 @@ template <int E, class Off>
 cudaError_t cols_fwd(const Problem& P, const ColArgs& A, float zq, cudaStream_t stream) {
   const unsigned blocks = (unsigned)((P.rows + kColC - 1) / kColC);
   const int threads = 32 * col_warps(P.n, E);
+  cudaError_t err;
   const bool mag = P.mode == TK_TOPKMAG;
   if (P.q4) {
-    if (mag) tk_cols_fwd_kernel<E, true, true, Off><<<blocks, threads, 0, stream>>>(P, A, zq);
-    else tk_cols_fwd_kernel<E, true, false, Off><<<blocks, threads, 0, stream>>>(P, A, zq);
+    if (mag) err = launch_overlapped(tk_cols_fwd_kernel<E, true, true, Off>, blocks, threads, 0, stream, P, A, zq);
+    else err = launch_overlapped(tk_cols_fwd_kernel<E, true, false, Off>, blocks, threads, 0, stream, P, A, zq);
   } else {
-    if (mag) tk_cols_fwd_kernel<E, false, true, Off><<<blocks, threads, 0, stream>>>(P, A, zq);
-    else tk_cols_fwd_kernel<E, false, false, Off><<<blocks, threads, 0, stream>>>(P, A, zq);
+    if (mag) err = launch_overlapped(tk_cols_fwd_kernel<E, false, true, Off>, blocks, threads, 0, stream, P, A, zq);
+    else err = launch_overlapped(tk_cols_fwd_kernel<E, false, false, Off>, blocks, threads, 0, stream, P, A, zq);
   }
-  return cudaGetLastError();
+  return err;
 }
 
 template <int E, class Off>
 cudaError_t cols_vjp(const Problem& P, const ColArgs& A, cudaStream_t stream) {
   const unsigned blocks = (unsigned)((P.rows + kColC - 1) / kColC);
   const int threads = 32 * col_warps(P.n, E);
+  cudaError_t err;
   if (P.q4) {
-    if (P.mode == TK_MASK) tk_cols_vjp_kernel<E, true, TK_MASK, Off><<<blocks, threads, 0, stream>>>(P, A);
-    else if (P.mode == TK_TOPK) tk_cols_vjp_kernel<E, true, TK_TOPK, Off><<<blocks, threads, 0, stream>>>(P, A);
-    else tk_cols_vjp_kernel<E, true, TK_TOPKMAG, Off><<<blocks, threads, 0, stream>>>(P, A);
+    if (P.mode == TK_MASK) err = launch_overlapped(tk_cols_vjp_kernel<E, true, TK_MASK, Off>, blocks, threads, 0, stream, P, A);
+    else if (P.mode == TK_TOPK) err = launch_overlapped(tk_cols_vjp_kernel<E, true, TK_TOPK, Off>, blocks, threads, 0, stream, P, A);
+    else err = launch_overlapped(tk_cols_vjp_kernel<E, true, TK_TOPKMAG, Off>, blocks, threads, 0, stream, P, A);
   } else {
-    if (P.mode == TK_MASK) tk_cols_vjp_kernel<E, false, TK_MASK, Off><<<blocks, threads, 0, stream>>>(P, A);
-    else if (P.mode == TK_TOPK) tk_cols_vjp_kernel<E, false, TK_TOPK, Off><<<blocks, threads, 0, stream>>>(P, A);
-    else tk_cols_vjp_kernel<E, false, TK_TOPKMAG, Off><<<blocks, threads, 0, stream>>>(P, A);
+    if (P.mode == TK_MASK) err = launch_overlapped(tk_cols_vjp_kernel<E, false, TK_MASK, Off>, blocks, threads, 0, stream, P, A);
+    else if (P.mode == TK_TOPK) err = launch_overlapped(tk_cols_vjp_kernel<E, false, TK_TOPK, Off>, blocks, threads, 0, stream, P, A);
+    else err = launch_overlapped(tk_cols_vjp_kernel<E, false, TK_TOPKMAG, Off>, blocks, threads, 0, stream, P, A);
   }
-  return cudaGetLastError();
+  return err;
 }
 
 // offsets inside a matrix fit 32 bits of bytes

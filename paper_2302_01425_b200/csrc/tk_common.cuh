@@ -72,6 +72,33 @@ inline int sm_count() {
   return cached[dev];
 }
 
+// ---------------------------------------------------------------- overlapped launches
+// A step is a chain of short kernels, and a launch takes about a microsecond in which the GPU idles.  Kernels launched by
+// launch_overlapped may start while the kernel before them in the stream still runs (their blocks take the places that it
+// has left), and wait for it to finish, memory included, in overlap_wait(): before that call they touch no global memory,
+// and what they read after it for the first time they read with plain loads (not through the read-only path, which assumes
+// data that nobody writes while the grid exists).  The kernel after them may start as soon as all their blocks have.
+__device__ __forceinline__ void overlap_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class... Params, class... Args>
+inline cudaError_t launch_overlapped(void (*kern)(Params...), dim3 blocks, dim3 threads, size_t smem, cudaStream_t stream,
+                                     Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = blocks;
+  cfg.blockDim = threads;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+
 // ---------------------------------------------------------------- keys
 // Order-preserving map float -> uint32 (larger float, larger integer).
 __device__ __forceinline__ uint32_t f2key(float x) {

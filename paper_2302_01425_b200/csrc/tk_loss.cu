@@ -22,8 +22,8 @@ __device__ __forceinline__ double loss_term(float x, float y, float lam_over_p, 
 }
 
 template <int PK, int TPR>      // TPR threads share a row: 32 (a warp) or 256 (the block)
-__global__ void __launch_bounds__(256) tk_loss_kernel(const float* __restrict__ theta,
-                                                      const int32_t* __restrict__ target, float* grad,
+__global__ void __launch_bounds__(256) tk_loss_kernel(const float* theta,
+                                                      const int32_t* target, float* grad,
                                                       float* __restrict__ loss, long long rows, int n,
                                                       float lam_over_p, float pm1, int vec4) {
   constexpr int RPB = 256 / TPR;
@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(256) tk_loss_kernel(const float* __restrict__ 
   const int lane = threadIdx.x % TPR;
   const long long row = (long long)blockIdx.x * RPB + threadIdx.x / TPR;
   const bool live = row < rows;
+  overlap_wait();
   double acc = 0.0;
   const float* x = theta + (live ? row : 0) * (long long)n;
   float* y = grad + (live ? row : 0) * (long long)n;
@@ -39,12 +40,12 @@ __global__ void __launch_bounds__(256) tk_loss_kernel(const float* __restrict__ 
       const float4* x4 = reinterpret_cast<const float4*>(x);
       const float4* y4 = reinterpret_cast<const float4*>(y);
       for (int i = lane; i < n / 4; i += TPR) {
-        const float4 a = __ldg(x4 + i), b = y4[i];
+        const float4 a = x4[i], b = y4[i];
         acc += loss_term<PK>(a.x, b.x, lam_over_p, pm1) + loss_term<PK>(a.y, b.y, lam_over_p, pm1);
         acc += loss_term<PK>(a.z, b.z, lam_over_p, pm1) + loss_term<PK>(a.w, b.w, lam_over_p, pm1);
       }
     } else {
-      for (int i = lane; i < n; i += TPR) acc += loss_term<PK>(__ldg(x + i), y[i], lam_over_p, pm1);
+      for (int i = lane; i < n; i += TPR) acc += loss_term<PK>(x[i], y[i], lam_over_p, pm1);
     }
   }
   acc = warp_sum(acc);
@@ -57,7 +58,7 @@ __global__ void __launch_bounds__(256) tk_loss_kernel(const float* __restrict__ 
   }
   // every read of this row's y* is complete (the shuffles, or the barrier, order it before this)
   if (live && lane == 0) {
-    const int t = target ? __ldg(target + row) : -1;
+    const int t = target ? target[row] : -1;
     if (t >= 0 && t < n) {
       acc -= (double)__ldg(x + t);
       y[t] = y[t] - 1.0f;
@@ -71,11 +72,9 @@ cudaError_t launch_pk(const float* theta, const int32_t* target, float* grad, fl
                       float lam_over_p, float pm1, int vec4, cudaStream_t stream) {
   if (n <= 2048) {
     const unsigned blocks = (unsigned)((rows + 7) / 8);
-    tk_loss_kernel<PK, 32><<<blocks, 256, 0, stream>>>(theta, target, grad, loss, rows, n, lam_over_p, pm1, vec4);
-  } else {
-    tk_loss_kernel<PK, 256><<<(unsigned)rows, 256, 0, stream>>>(theta, target, grad, loss, rows, n, lam_over_p, pm1, vec4);
+    return launch_overlapped(tk_loss_kernel<PK, 32>, blocks, 256, 0, stream, theta, target, grad, loss, rows, n, lam_over_p, pm1, vec4);
   }
-  return cudaGetLastError();
+  return launch_overlapped(tk_loss_kernel<PK, 256>, (unsigned)rows, 256, 0, stream, theta, target, grad, loss, rows, n, lam_over_p, pm1, vec4);
 }
 
 }  // namespace

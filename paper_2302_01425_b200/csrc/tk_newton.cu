@@ -110,6 +110,8 @@ struct NtIO {
   }
   // the four words of chunk c as they are in memory (a chunk past the row re-reads the row's start:
   // no load depends on a test, so the loads of a lane are all in flight at once)
+  // AGAIN: the row has been read before, the read-only path may be taken
+  template <bool AGAIN>
   __device__ __forceinline__ void load_raw(int c, float (&x)[4]) const {
     const int p0 = pos(c);
     if (STAGED) {
@@ -122,13 +124,14 @@ struct NtIO {
       const int pc = p0 < n ? p0 : 0;
       x[0] = x[1] = x[2] = x[3] = 0.0f;
       if (!TK_IN_BOUNDS(first + pc, 4, extent, status)) return;
-      const float4 v = __ldg(reinterpret_cast<const float4*>(src + pc));
+      const float4* at = reinterpret_cast<const float4*>(src + pc);
+      const float4 v = AGAIN ? __ldg(at) : *at;
       x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int pc = p0 + j < n ? p0 + j : 0;
-        x[j] = TK_IN_BOUNDS(first + pc, 1, extent, status) ? __ldg(src + pc) : 0.0f;
+        x[j] = TK_IN_BOUNDS(first + pc, 1, extent, status) ? (AGAIN ? __ldg(src + pc) : src[pc]) : 0.0f;
       }
     }
   }
@@ -144,7 +147,7 @@ struct NtIO {
     }
   }
   __device__ __forceinline__ void load(int c, float (&x)[4]) const {
-    load_raw(c, x);
+    load_raw<true>(c, x);
     mask(c, x);
   }
   __device__ __forceinline__ void store(int c, const float (&y)[4]) const {
@@ -208,6 +211,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
   io.first = row_c * (long long)n; io.extent = P.rows * (long long)n; io.status = P.status;
   io.lane_in_warp = lane;
   io.span4 = nullptr;
+  overlap_wait();
   if (STAGED) {
     // ---- stage the warp's rows (contiguous in memory) in its tile, row stride G * E
     constexpr int RS = G * E;
@@ -221,10 +225,10 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
         const float4* s4 = reinterpret_cast<const float4*>(src);
         float4* t4 = reinterpret_cast<float4*>(tile);
         for (int v = lane; 4 * v < total; v += 32)
-          if (TK_IN_BOUNDS(row0 * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(4 * v, 4, 32 * E, P.status)) t4[v] = __ldg(s4 + v);
+          if (TK_IN_BOUNDS(row0 * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(4 * v, 4, 32 * E, P.status)) t4[v] = s4[v];
       } else {
         for (int i = lane; i < total; i += 32)
-          if (TK_IN_BOUNDS(row0 * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(i, 1, 32 * E, P.status)) tile[i] = __ldg(src + i);
+          if (TK_IN_BOUNDS(row0 * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(i, 1, 32 * E, P.status)) tile[i] = src[i];
       }
     } else {
       for (int r = 0; r < rows_here; ++r) {
@@ -232,10 +236,10 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
           const float4* s4 = reinterpret_cast<const float4*>(src + (long long)r * n);
           float4* t4 = reinterpret_cast<float4*>(tile + r * RS);
           for (int v = lane; 4 * v < n; v += 32)
-            if (TK_IN_BOUNDS((row0 + r) * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(r * RS + 4 * v, 4, 32 * E, P.status)) t4[v] = __ldg(s4 + v);
+            if (TK_IN_BOUNDS((row0 + r) * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(r * RS + 4 * v, 4, 32 * E, P.status)) t4[v] = s4[v];
         } else {
           for (int i = lane; i < n; i += 32)
-            if (TK_IN_BOUNDS((row0 + r) * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(r * RS + i, 1, 32 * E, P.status)) tile[r * RS + i] = __ldg(src + (long long)r * n + i);
+            if (TK_IN_BOUNDS((row0 + r) * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(r * RS + i, 1, 32 * E, P.status)) tile[r * RS + i] = src[(long long)r * n + i];
         }
       }
     }
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     float x4[4];
-    io.load_raw(c, x4);
+    io.template load_raw<false>(c, x4);
 #pragma unroll
     for (int j = 0; j < 4; ++j) d[4 * c + j] = MAG ? fabsf(x4[j]) : x4[j];
   }
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
   float lo = -FLT_MAX, hi = FLT_MAX;
   if (KSEL == 0) {
     // sums about the row's first key: mean and spread of the keys
-    const float x0 = MAG ? 0.0f : __ldg(io.src);
+    const float x0 = MAG ? 0.0f : *io.src;
     float v[2] = {0.f, 0.f};
     uint32_t nnz = 0;                          // phi even: keys above 0
     if (full) {
@@ -566,8 +570,7 @@ cudaError_t nt_launch(const Problem& P, float zq, cudaStream_t stream) {
   // rows in flight on the whole GPU: the distance the prefetch looks ahead
   const long long wave = (long long)sm_count() * nt_min_blocks(E, W, Q4, STAGED, G) * rows_per_block;
   const int pf_rows = (int)(wave < 0x7fffffff ? wave : 0);
-  kern<<<blocks, BW * 32, smem, stream>>>(P, zq, pf_rows);
-  return cudaGetLastError();
+  return launch_overlapped(kern, blocks, BW * 32, smem, stream, P, zq, pf_rows);
 }
 
 // KS: the shape also has the variants that track the k + 1 largest keys (k <= 2, phi = x)

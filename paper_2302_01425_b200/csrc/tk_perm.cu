@@ -45,10 +45,11 @@ __global__ void __launch_bounds__(RankGeom<G, W>::THREADS, (W == 1 ? 6 : (W >= 1
   int* work = reinterpret_cast<int*>(sm + R * NP);
   const bool mag = P.mode == TK_TOPKMAG;
 
+  overlap_wait();
   float x[E], r[E];
   bool bad = false;
 #pragma unroll
-  for (int i = 0; i < E; ++i) x[i] = __ldg(P.theta + first + min(lig + T * i, n - 1));
+  for (int i = 0; i < E; ++i) x[i] = P.theta[first + min(lig + T * i, n - 1)];
 #pragma unroll
   for (int i = 0; i < E; ++i) bad |= !(fabsf(x[i]) < INFINITY);
   auto key_of = [&](float v) -> float {
@@ -105,8 +106,7 @@ cudaError_t pm_launch(const PermArgs& P, cudaStream_t stream) {
     }
   }
   const unsigned blocks = (unsigned)((P.rows + rows_per_block - 1) / rows_per_block);
-  tk_perm_kernel<G, W><<<blocks, Geom::THREADS, smem, stream>>>(P);
-  return cudaGetLastError();
+  return launch_overlapped(tk_perm_kernel<G, W>, blocks, Geom::THREADS, smem, stream, P);
 }
 
 }  // namespace

@@ -336,15 +336,16 @@ __global__ void __launch_bounds__(kRowsThreads, E <= 16 ? 6 : 3) tk_rows_kernel(
   int flags = 0;
 
   // elements 4 h .. 4 h + 3 of the lane's E consecutive elements of a row (zeros past the row's end)
+  overlap_wait();
   auto load4 = [&](const float* base, bool live, int h, float (&v4)[4]) {
     const int e0 = E * lig + 4 * h;
     if (P.vec4) {
       float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (live && e0 < n) q = __ldg(reinterpret_cast<const float4*>(base) + (e0 >> 2));
+      if (live && e0 < n) q = reinterpret_cast<const float4*>(base)[e0 >> 2];
       v4[0] = q.x; v4[1] = q.y; v4[2] = q.z; v4[3] = q.w;
     } else {
 #pragma unroll
-      for (int c4 = 0; c4 < 4; ++c4) v4[c4] = (live && e0 + c4 < n) ? __ldg(base + e0 + c4) : 0.0f;
+      for (int c4 = 0; c4 < 4; ++c4) v4[c4] = (live && e0 + c4 < n) ? base[e0 + c4] : 0.0f;
     }
   };
 
@@ -582,20 +583,16 @@ cudaError_t launch_rows_gb(const Problem& P, cudaStream_t stream) {
   if (P.qm1 > 0.0f) {                          // any other q: rows of up to 128 elements, not the magnitude mode
     if constexpr (G <= 16 && E <= 16) {
       if (mag) return cudaErrorInvalidValue;
-      tk_rows_kernel<G, E, B, 2, false><<<blocks, kRowsThreads, 0, stream>>>(P);
-      return cudaGetLastError();
+      return launch_overlapped(tk_rows_kernel<G, E, B, 2, false>, blocks, kRowsThreads, 0, stream, P);
     } else {
       return cudaErrorInvalidValue;
     }
   }
-  if (P.q4) {
-    if (mag) tk_rows_kernel<G, E, B, 1, true><<<blocks, kRowsThreads, 0, stream>>>(P);
-    else tk_rows_kernel<G, E, B, 1, false><<<blocks, kRowsThreads, 0, stream>>>(P);
-  } else {
-    if (mag) tk_rows_kernel<G, E, B, 0, true><<<blocks, kRowsThreads, 0, stream>>>(P);
-    else tk_rows_kernel<G, E, B, 0, false><<<blocks, kRowsThreads, 0, stream>>>(P);
-  }
-  return cudaGetLastError();
+  if (P.q4)
+    return mag ? launch_overlapped(tk_rows_kernel<G, E, B, 1, true>, blocks, kRowsThreads, 0, stream, P)
+               : launch_overlapped(tk_rows_kernel<G, E, B, 1, false>, blocks, kRowsThreads, 0, stream, P);
+  return mag ? launch_overlapped(tk_rows_kernel<G, E, B, 0, true>, blocks, kRowsThreads, 0, stream, P)
+             : launch_overlapped(tk_rows_kernel<G, E, B, 0, false>, blocks, kRowsThreads, 0, stream, P);
 }
 
 // warps below which a launch leaves SMs short of work: 24 per SM

@@ -209,10 +209,11 @@ __global__ void __launch_bounds__(RankGeom<G, W>::THREADS, (W == 1 ? 5 : (W >= 1
   float* ys = work + rl * 2 * SwGeom<G, W>::VN;
   const float* x_row = P.theta + first;
 
+  overlap_wait();
   float key[E], r[E];
   bool bad = false;
 #pragma unroll
-  for (int i = 0; i < E; ++i) key[i] = __ldg(x_row + min(lig + T * i, n - 1));
+  for (int i = 0; i < E; ++i) key[i] = x_row[min(lig + T * i, n - 1)];
 #pragma unroll
   for (int i = 0; i < E; ++i) bad |= !(fabsf(key[i]) < INFINITY);
 #pragma unroll
@@ -268,10 +269,9 @@ cudaError_t sw_launch(const Problem& P, int lo, int hi, cudaStream_t stream) {
   using Geom = RankGeom<G, W>;
   constexpr int rows_per_block = Geom::TEAMS * Geom::R;
   const unsigned blocks = (unsigned)((P.rows + rows_per_block - 1) / rows_per_block);
-  if (P.q4) tk_sweeps_kernel<G, W, true, false><<<blocks, Geom::THREADS, 0, stream>>>(P, lo, hi);
-  else if (P.mode == TK_TOPKMAG) tk_sweeps_kernel<G, W, false, true><<<blocks, Geom::THREADS, 0, stream>>>(P, lo, hi);
-  else tk_sweeps_kernel<G, W, false, false><<<blocks, Geom::THREADS, 0, stream>>>(P, lo, hi);
-  return cudaGetLastError();
+  if (P.q4) return launch_overlapped(tk_sweeps_kernel<G, W, true, false>, blocks, Geom::THREADS, 0, stream, P, lo, hi);
+  if (P.mode == TK_TOPKMAG) return launch_overlapped(tk_sweeps_kernel<G, W, false, true>, blocks, Geom::THREADS, 0, stream, P, lo, hi);
+  return launch_overlapped(tk_sweeps_kernel<G, W, false, false>, blocks, Geom::THREADS, 0, stream, P, lo, hi);
 }
 
 // the ranks that `sweeps` sweeps can change, first of a pair of C1 onwards

@@ -162,15 +162,15 @@ __device__ __forceinline__ void long_load(const Problem& P, long long row, int s
     T.x[j] = T.g[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (P.vec4) {                               // n % 4 == 0 and aligned rows: 128-bit loads
       if (e < n) {
-        T.x[j] = __ldg(reinterpret_cast<const float4*>(x_row + e));
-        T.g[j] = __ldg(reinterpret_cast<const float4*>(g_row + e));
+        T.x[j] = *reinterpret_cast<const float4*>(x_row + e);
+        T.g[j] = *reinterpret_cast<const float4*>(g_row + e);
       }
     } else {
       float* xs = reinterpret_cast<float*>(&T.x[j]);
       float* gs = reinterpret_cast<float*>(&T.g[j]);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (e + q < n) { xs[q] = __ldg(x_row + e + q); gs[q] = __ldg(g_row + e + q); }
+        if (e + q < n) { xs[q] = x_row[e + q]; gs[q] = g_row[e + q]; }
     }
   }
 }
@@ -181,6 +181,7 @@ __global__ void __launch_bounds__(256) tk_vjp_long_partial(const Problem P, doub
   const Math M = long_math<Q4, MAG>(P);
   const long long row = blockIdx.y;
   const int tile = blockIdx.x, t = threadIdx.x, start = tile * kLongTile;
+  overlap_wait();
   LongTile T;
   long_load(P, row, start, T);
   const RowCtx c = load_ctx(P, M, row);
@@ -210,6 +211,7 @@ __global__ void __launch_bounds__(256) tk_vjp_long_finish(const Problem P, const
   const Math M = long_math<Q4, MAG>(P);
   const long long row = blockIdx.y;
   const int tile = blockIdx.x, t = threadIdx.x, n = P.n, start = tile * kLongTile;
+  overlap_wait();
   LongTile T;
   long_load(P, row, start, T);
   const RowCtx c = load_ctx(P, M, row);
@@ -250,9 +252,9 @@ cudaError_t launch_vjp_state_long(const Problem& P, void* scratch, cudaStream_t 
   const dim3 grid((unsigned)tiles, (unsigned)P.rows);
   double2* partial = static_cast<double2*>(scratch);
   auto run = [&](auto part, auto fin) {
-    part<<<grid, 256, 0, stream>>>(P, partial, tiles);
-    fin<<<grid, 256, 0, stream>>>(P, partial, tiles);
-    return cudaGetLastError();
+    const cudaError_t err = launch_overlapped(part, grid, dim3(256), 0, stream, P, partial, tiles);
+    if (err != cudaSuccess) return err;
+    return launch_overlapped(fin, grid, dim3(256), 0, stream, P, partial, tiles);
   };
   const bool mag = P.mode == TK_TOPKMAG;
   if (P.q4) return mag ? run(tk_vjp_long_partial<true, true>, tk_vjp_long_finish<true, true>)

@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk
   const float* g_row = P.gout + row_c * (long long)n;
   float* o_row = P.out + row_c * (long long)n;
 
+  overlap_wait();
   // ---- theta and g: every load is unconditional (a chunk past the row re-reads its start)
   float x[E], g[E];
 #pragma unroll
@@ -101,8 +102,8 @@ __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk
       const int pc = p0 < n ? p0 : 0;
       float4 xv = make_float4(0.f, 0.f, 0.f, 0.f), gv = xv;
       if (TK_IN_BOUNDS(row_c * (long long)n + pc, 4, P.rows * (long long)n, P.status)) {
-        xv = __ldg(reinterpret_cast<const float4*>(x_row + pc));
-        gv = __ldg(reinterpret_cast<const float4*>(g_row + pc));
+        xv = *reinterpret_cast<const float4*>(x_row + pc);
+        gv = *reinterpret_cast<const float4*>(g_row + pc);
       }
       x[4 * c] = xv.x; x[4 * c + 1] = xv.y; x[4 * c + 2] = xv.z; x[4 * c + 3] = xv.w;
       g[4 * c] = gv.x; g[4 * c + 1] = gv.y; g[4 * c + 2] = gv.z; g[4 * c + 3] = gv.w;
@@ -111,8 +112,8 @@ __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk
       for (int j = 0; j < 4; ++j) {
         const int pc = p0 + j < n ? p0 + j : 0;
         const bool okb = TK_IN_BOUNDS(row_c * (long long)n + pc, 1, P.rows * (long long)n, P.status);
-        x[4 * c + j] = okb ? __ldg(x_row + pc) : 0.0f;
-        g[4 * c + j] = okb ? __ldg(g_row + pc) : 0.0f;
+        x[4 * c + j] = okb ? x_row[pc] : 0.0f;
+        g[4 * c + j] = okb ? g_row[pc] : 0.0f;
       }
     }
   }
@@ -208,8 +209,7 @@ cudaError_t vt_launch(const Problem& P, cudaStream_t stream) {
   constexpr long long rows_per_block = (long long)TEAMS * (W > 1 ? 1 : 32 / G);
   if (CL == 1) {
     const unsigned blocks = (unsigned)((P.rows + rows_per_block - 1) / rows_per_block);
-    tk_vjp_team_kernel<G, E, W, QM, MODE, CL><<<blocks, BW * 32, smem, stream>>>(P);
-    return cudaGetLastError();
+    return launch_overlapped(tk_vjp_team_kernel<G, E, W, QM, MODE, CL>, blocks, BW * 32, smem, stream, P);
   }
   // CL thread blocks per row, launched as a cluster
   if (P.rows > 0x3fffffffLL) return cudaErrorInvalidValue;
@@ -218,13 +218,15 @@ cudaError_t vt_launch(const Problem& P, cudaStream_t stream) {
   cfg.blockDim = dim3(BW * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CL;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, tk_vjp_team_kernel<G, E, W, QM, MODE, CL>, P);
 }
 

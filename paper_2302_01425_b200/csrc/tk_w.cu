@@ -127,7 +127,7 @@ struct WGeom {
 
 template <int E, int G, int W, bool Q4, bool VJP>
 __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN_BLOCKS)
-    tk_w_kernel(const Problem P, const float* __restrict__ w_all, const int w_shared) {
+    tk_w_kernel(const Problem P, const float* w_all, const int w_shared) {
   static_assert(W == 1 || G == 32, "several warps per row: every lane of them belongs to the row");
   constexpr int T = G * W, R = W > 1 ? 1 : 32 / G;                // lanes per row, rows per team
   constexpr int N = T * E, NP = N + T;                            // padded row length, its slots
@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
   const uint32_t magic = n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u;
   auto row_of = [&](int e) -> int { return R == 1 ? 0 : (n > 1 ? (int)__umulhi((uint32_t)e, magic) : e); };
 
+  overlap_wait();
   // ---- theta as it lies in memory, w by rank (in the keys' array, which is free until the sort is done).  Every
   // load is unconditional (past the end the last element again), so the loads of a lane are all in flight at once
   bool bad = false;
@@ -185,18 +186,18 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
     float v[E];
     const float* src = P.theta + first;
 #pragma unroll
-    for (int it = 0; it < E; ++it) v[it] = __ldg(src + min(tid + it * TL, total - 1));
+    for (int it = 0; it < E; ++it) v[it] = src[min(tid + it * TL, total - 1)];
 #pragma unroll
     for (int it = 0; it < E; ++it) {
       bad |= !(fabsf(v[it]) < INFINITY);
       if (tid + it * TL < total) xs[tid + it * TL] = v[it];
     }
     if (w_shared) {
-      for (int i = tid; i < n; i += TL) s[wp<E>(i)] = __ldg(w_all + i);
+      for (int i = tid; i < n; i += TL) s[wp<E>(i)] = w_all[i];
     } else {
       src = w_all + first;
 #pragma unroll
-      for (int it = 0; it < E; ++it) v[it] = __ldg(src + min(tid + it * TL, total - 1));
+      for (int it = 0; it < E; ++it) v[it] = src[min(tid + it * TL, total - 1)];
 #pragma unroll
       for (int it = 0; it < E; ++it) {
         const int e = tid + it * TL, r = row_of(e);
@@ -545,7 +546,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
       rk[it] = rr * NP + wp<E>(rank);
     }
 #pragma unroll
-    for (int it = 0; it < E; ++it) gv[it] = __ldg(P.gout + first + min(tid + it * TL, total - 1));
+    for (int it = 0; it < E; ++it) gv[it] = P.gout[first + min(tid + it * TL, total - 1)];
     tie = W > 1 ? __syncthreads_or(tie) != 0 : __any_sync(0xffffffffu, tie);
     if (tie) {
       // runs of equal keys: ranks in index order.  One warp walks the elements 32 at a time; cnt: how many of a
@@ -691,8 +692,7 @@ cudaError_t w_launch(const Problem& P, const float* w, int w_shared, cudaStream_
     }
   }
   const unsigned blocks = (unsigned)((P.rows + rows_per_block - 1) / rows_per_block);
-  kern<<<blocks, WGeom<E, W, Q4>::THREADS, smem, stream>>>(P, w, w_shared);
-  return cudaGetLastError();
+  return launch_overlapped(kern, blocks, WGeom<E, W, Q4>::THREADS, smem, stream, P, w, w_shared);
 }
 
 // Lanes and warps of a row of n elements with E ranks per lane.
