@@ -77,10 +77,18 @@ inline int sm_count() {
 // launch_overlapped may start while the kernel before them in the stream still runs (their blocks take the places that it
 // has left), and wait for it to finish, memory included, in overlap_wait(): before that call they touch no global memory,
 // and what they read after it for the first time they read with plain loads (not through the read-only path, which assumes
-// data that nobody writes while the grid exists).  The kernel after them may start as soon as all their blocks have.
+// data that nobody writes while the grid exists).  The kernel after them may start once all their blocks have called
+// overlap_next() (or ended).  Where that is matters: blocks of the next grid that settle while most of this one's are still
+// at work crowd the SMs that have room, and their share of the work stays there.
+// After the row has been read and the starting guess is known was the best place for the Newton kernel and its VJP
+// (forward + VJP, us: at the kernel's start / there: 10007 x 60 p = 4/3 14.0 / 12.4, 16384 x 32 k = 4 22.1 / 13.6,
+// 4000 x 200 17.4 / 12.6, 4096 x 512 17.6 / 16.0; 16384 x 64 k = 2 7.3 / 7.6); rows in whole waves do not care.
 __device__ __forceinline__ void overlap_wait() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__device__ __forceinline__ void overlap_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <class... Params, class... Args>

@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
   io.first = row_c * (long long)n; io.extent = P.rows * (long long)n; io.status = P.status;
   io.lane_in_warp = lane;
   io.span4 = nullptr;
+  if (KSEL != 0) overlap_next();               // k <= 2: no iteration to speak of, the next grid may queue at once
   overlap_wait();
   if (STAGED) {
     // ---- stage the warp's rows (contiguous in memory) in its tile, row stride G * E
@@ -371,6 +372,8 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
     if (pf_rows > 0 && first < end && lane * 32 < R * n)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(P.theta + first));
   }
+
+  if (KSEL == 0) overlap_next();
 
   // ---- the iteration
   int passes = 0;

@@ -181,6 +181,7 @@ __global__ void __launch_bounds__(256) tk_vjp_long_partial(const Problem P, doub
   const Math M = long_math<Q4, MAG>(P);
   const long long row = blockIdx.y;
   const int tile = blockIdx.x, t = threadIdx.x, start = tile * kLongTile;
+  overlap_next();
   overlap_wait();
   LongTile T;
   long_load(P, row, start, T);
@@ -211,6 +212,7 @@ __global__ void __launch_bounds__(256) tk_vjp_long_finish(const Problem P, const
   const Math M = long_math<Q4, MAG>(P);
   const long long row = blockIdx.y;
   const int tile = blockIdx.x, t = threadIdx.x, n = P.n, start = tile * kLongTile;
+  overlap_next();
   overlap_wait();
   LongTile T;
   long_load(P, row, start, T);

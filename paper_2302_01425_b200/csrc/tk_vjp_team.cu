@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk
     AD[0] = fmaf(dr * chi, gv, AD[0]);
     AD[1] += dr;
   }
+  overlap_next();
   float ratio = 0.0f, delta = 0.0f;
   if (__any_sync(0xffffffffu, has_block)) {    // the warps of a row agree: same row state
     uint32_t none = 0;
