@@ -165,9 +165,16 @@ size_t tk_workspace_bytes(int64_t rows, int64_t n, int64_t k, double p, int mode
   return tk::long_workspace_bytes(rows, (int)n);
 }
 
+// the smooth top-k loss (tk_topk_loss) on top of a relaxed mask; *done: the forward kernel has made it
+struct LossArgs {
+  const int32_t* target;
+  float* loss;
+  bool done;
+};
+
 // hard: out receives the hard operator (straight-through); *hard_done: it has, else the caller makes it from perm_out.
 static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_t k, double p, double lambda, int mode,
-                             float* out, const tk_opts* opts, tk_stream stream, bool hard, bool* hard_done) {
+                             float* out, const tk_opts* opts, tk_stream stream, bool hard, bool* hard_done, LossArgs* loss) {
   int q4 = 0;
   double qm1 = 0.0;
   tk_status s = check_common(theta, rows, n, k, p, lambda, mode, &q4, &qm1);
@@ -191,16 +198,19 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
   P.what = tk::W_FWD;
   if (opts) { P.perm_out = opts->perm_out; P.state_out = opts->state_out; P.status = opts->status_out; }
   P.vec4 = (n % 4 == 0) && aligned16(theta) && aligned16(out);
+  tk::Problem L = P;                            // what the threshold form is asked for
+  if (loss) { L.loss = loss->loss; L.target = loss->target; }
   // A permutation from AUTO: the order comes from the keys-only sort, the relaxed values and the row state from the
   // threshold form, which needs no order.  One kernel that sorts 64-bit words and solves on them (and another that makes
   // the hard output) stays faster up to 32 elements only: 699050 x 24, p = 2: 269 us and 270; 262144 x 64: 221 and 118;
   // 4194 x 4000: 420 and 265.  A hard output needs the row state alone.
   if (solver == TK_SOLVER_AUTO && P.perm_out && qm1 == 0.0 && n > 32 && n <= tk::perm_max_n()) {
-    tk::Problem F = P;
+    tk::Problem F = L;
     F.perm_out = nullptr;
     if (hard) { F.out = nullptr; *hard_done = true; }
     if (!hard || F.state_out) {
       if (tk::launch_newton(F, (cudaStream_t)stream) != cudaSuccess) return TK_ERR_CUDA;
+      if (loss) loss->done = true;
     }
     return tk::launch_perm(theta, rows, (int)n, (int)k, mode, P.perm_out, nullptr, hard ? out : nullptr, P.status,
                            (cudaStream_t)stream) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
@@ -211,7 +221,8 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
   const bool by_threshold = (solver == TK_SOLVER_THRESHOLD || (solver == TK_SOLVER_AUTO && n > (q4 ? 16 : 8))) &&
                             qm1 == 0.0 && P.perm_out == nullptr && n <= tk::newton_max_n();
   if (by_threshold) {
-    cudaError_t en = tk::launch_newton(P, (cudaStream_t)stream);
+    cudaError_t en = tk::launch_newton(L, (cudaStream_t)stream);
+    if (loss) loss->done = true;
     return en == cudaSuccess ? TK_OK : TK_ERR_CUDA;
   }
   // A few very long rows (the pruning row): the same iteration with the row streamed from L2, all SMs on
@@ -276,7 +287,7 @@ tk_status tk_fwd_ex(const float* theta, int64_t rows, int64_t n, int64_t k, doub
   if (st && rows > 0 && opts->perm_out == nullptr) return TK_ERR_INVALID_ARG;
   if (st && opts->solver == TK_SOLVER_THRESHOLD) return TK_ERR_UNSUPPORTED;
   bool hard_done = false;
-  tk_status s = fwd_relaxed(theta, rows, n, k, p, lambda, mode, out, opts, stream, st, &hard_done);
+  tk_status s = fwd_relaxed(theta, rows, n, k, p, lambda, mode, out, opts, stream, st, &hard_done, nullptr);
   if (s != TK_OK || !st || rows == 0 || hard_done) return s;
   // the relaxed pass has left the permutation (and the row state); the hard operator replaces its output
   cudaError_t e = tk::launch_hard(theta, opts->perm_out, out, rows, (int)n, (int)k, mode, (cudaStream_t)stream);
@@ -392,9 +403,12 @@ tk_status tk_topk_loss(const float* theta, const int32_t* target, int64_t rows, 
   if (s != TK_OK) return s;
   if (rows == 0) return TK_OK;
   if (loss == nullptr || grad == nullptr || (opts && opts->flags)) return TK_ERR_INVALID_ARG;
-  // the relaxed mask y* into grad (every check of the forward pass applies), then one pass over (theta, y*)
-  s = tk_fwd_ex(theta, rows, n, k, p, lambda, TK_MASK, grad, opts, stream);
-  if (s != TK_OK) return s;
+  // the relaxed mask y* into grad (every check of the forward pass applies), then one pass over (theta, y*); the threshold
+  // form makes the loss while the row is in its registers (8192 x 1000, p = 2: 38 us as two kernels, 31 as one)
+  LossArgs args = {target, loss, false};
+  bool hard_done = false;
+  s = fwd_relaxed(theta, rows, n, k, p, lambda, TK_MASK, grad, opts, stream, false, &hard_done, &args);
+  if (s != TK_OK || args.done) return s;
   const int vec4 = (n % 4 == 0) && aligned16(theta) && aligned16(grad);
   cudaError_t e = tk::launch_loss(theta, target, grad, loss, rows, (int)n, p, lambda, q4, qm1, vec4,
                                   (cudaStream_t)stream);

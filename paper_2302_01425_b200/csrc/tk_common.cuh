@@ -20,10 +20,16 @@ constexpr int kLongTile = 4096;   // elements per thread block in the kernels fo
 
 struct Problem {
   const float* theta;
-  const float* gout;        // cotangent (VJP only)
+  union {
+    const float* gout;      // cotangent (VJP only)
+    const int32_t* target;  // forward pass with a loss: the class of each row (may be null, or outside the row: no target)
+  };
   float* out;               // operator output (forward) or grad_theta (VJP)
   int32_t* perm_out;
-  float* sorted_out;
+  union {
+    float* sorted_out;      // sorting kernels
+    float* loss;            // Newton kernel: when set, out receives mask - t and loss[r] the smooth top-k loss
+  };
   tk_rowstate* state_out;
   const tk_rowstate* state_in;
   int32_t* status;

@@ -3,8 +3,8 @@
 // with phi(x) = x (Prop. "Relaxed operator": the maximiser is the relaxed top-k
 // mask y*, and grad_1 f = y*), R(y) = (lambda/p) sum y_i^p, t one-hot.
 //
-// The forward pass has already written y* into `grad`; this pass reads x and y*
-// once, reduces  sum_i y_i (x_i - (lambda/p) y_i^(p-1))  per row (most y_i are
+// For the forward passes that do not make the loss themselves (the Newton kernel does): y* is
+// in `grad`; this pass reads x and y* once, reduces  sum_i y_i (x_i - (lambda/p) y_i^(p-1))  per row (most y_i are
 // exactly 0 or 1), subtracts x[target] and turns y* into the gradient y* - t.
 #include "tk_common.cuh"
 

@@ -73,6 +73,13 @@ __device__ __forceinline__ void nt_top3(float x, float& m1, float& m2, float& m3
   m3 = fmaxf(m3, r2);
 }
 
+// the larger of the two, NaN if either is
+__device__ __forceinline__ float nt_max_nan(float x, float y) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
+  return r;
+}
+
 // threads per block, and the blocks per SM the register budget is set for: 24 warps of 80 registers with
 // up to 32 keys per lane, 16 warps of 128 registers with 64
 constexpr int nt_threads(int W) { return team_threads(W); }
@@ -171,11 +178,271 @@ struct NtIO {
 __device__ __forceinline__ void nt_fence() { asm volatile("" ::: "memory"); }
 
 
+// what is made of the root; NT_MAG: phi(x) = x^2/2, keys |theta|
+enum NtWhat { NT_MASK, NT_TOPK, NT_LOSS, NT_MAG };
+
+// Where a thread works.  Built again after the iteration (and for a new pivot) from the special registers: the registers that
+// hold row addresses and indices are the iteration's then, which spilled without them (kept / built again, us: 131072 x 512,
+// p = 4/3 157 / 151, 262144 x 64 37 / 33, 8192 x 8192 141 / 129, 2048 x 32768, p = 4/3 213 / 204).  Rows of four warps run
+// slower that way, without spilling either way (16384 x 4096, p = 4/3 155 / 173, p = 2 118 / 132): kept there.
+template <int E, int W>
+struct NtRebuild {
+  static constexpr bool v = W != 4;
+};
+
+template <int G, int E, int W, bool STAGED>
+struct NtPlace {
+  int lane, warp, team, wit, lig;
+  long long row0, row;                         // the team's first row, this lane's row
+  NtIO<G, E, W, STAGED> io;
+  __device__ __forceinline__ NtPlace(const Problem& P, float* smem, unsigned tid, unsigned cta) {
+    constexpr int BW = kNtWarps > W ? kNtWarps : W, TEAMS = BW / W, R = W > 1 ? 1 : 32 / G;
+    lane = tid & 31; warp = tid >> 5;
+    team = warp / W; wit = warp % W;
+    row0 = ((long long)cta * TEAMS + team) * R;
+    lig = lane % G;
+    row = row0 + lane / G;
+    io.n = P.n; io.vec4 = P.vec4; io.row_ok = row < P.rows;
+    io.tl = W > 1 ? wit * 32 + lane : lig;
+    io.rot = nt_rot<E>(lane);
+    // a group past the last row works on the last row again and stores nothing
+    const long long row_c = io.row_ok ? row : P.rows - 1;
+    io.src = P.theta + row_c * (long long)P.n;
+    io.dst = P.out + row_c * (long long)P.n;
+    io.first = row_c * (long long)P.n; io.extent = P.rows * (long long)P.n; io.status = P.status;
+    io.lane_in_warp = lane;
+    io.span4 = STAGED ? reinterpret_cast<float4*>(smem + warp * (32 * E) + lane * E) : nullptr;
+  }
+};
+__device__ __forceinline__ unsigned nt_tid() {
+  unsigned v;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(v));
+  return v;
+}
+__device__ __forceinline__ unsigned nt_cta() {
+  unsigned v;
+  asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(v));
+  return v;
+}
+
+// What follows the iteration: the row state, and what WHAT asks for from the keys in the registers.
+template <int G, int E, int W, bool Q4, bool STAGED, NtWhat WHAT>
+__device__ __forceinline__ void nt_finish(const Problem& P, const NtPlace<G, E, W, STAGED>& at, NtRow& S, float (&d)[E],
+                                          float wid, bool early, bool bad, int phase, float* smem) {
+  constexpr bool MAG = WHAT == NT_MAG;
+  constexpr int BW = kNtWarps > W ? kNtWarps : W, TEAMS = BW / W, R = W > 1 ? 1 : 32 / G, CH = E / 4;
+  const int lane = at.lane, warp = at.warp, team = at.team, wit = at.wit, lig = at.lig;
+  const long long row0 = at.row0, row = at.row;
+  const NtIO<G, E, W, STAGED>& io = at.io;
+  const bool row_ok = io.row_ok;
+  const int n = P.n, k = P.k;
+  const float lam = P.lam, inv_lam = P.inv_lam;
+  float* red = smem + (STAGED ? BW * 32 * E : 0) + team * (2 * W * 4);
+  const int bar = 1 + team;
+  int flags = 0;
+  if (!S.done) {                               // cap reached: keep the last point, say so
+    flags |= TK_FLAG_NOT_CONVERGED;
+    S.a0 = k; S.b0 = k;
+  }
+  if (S.b0 <= S.a0) { S.a0 = k; S.b0 = k; }
+  const bool block = S.b0 > S.a0;
+  if (MAG) wid = nt_width<Q4, true>(S.piv + S.off, lam);   // of the point the last pass classified at
+
+  // ---- row state.  Without a block the VJP classifies by key >= pivot: any value above the
+  // (k+1)-th largest key and not above the k-th serves; tau + lambda/2 is one when lambda is
+  // resolved at the keys' magnitude, else the smallest capped key is looked up.
+  float piv_state = S.piv, off_state = S.off;
+  {
+    const bool want_p = row_ok && !block && !early;
+    const bool safe = wid > 9.6e-7f * (fabsf(S.piv) + fabsf(S.off));
+    const bool scan = want_p && !safe;
+    if (__any_sync(0xffffffffu, scan)) {       // uniform over the warps of a row: they hold the same S
+      float cmin = INFINITY;
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        float x4[4];
+        io.load(c, x4);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (d[4 * c + j] - S.off >= wid) cmin = fminf(cmin, MAG ? fabsf(x4[j]) : x4[j]);
+        if ((c & 3) == 3) nt_fence();
+      }
+      cmin = team_gmin<G>(cmin);
+      if (W > 1) {
+        float* rb = red + (phase & 1) * (W * 4);
+        ++phase;
+        if (lane == 0 && TK_IN_BOUNDS(team * (2 * W * 4) + ((phase - 1) & 1) * (W * 4) + wit * 4, 1, TEAMS * 2 * W * 4, P.status)) rb[wit * 4] = cmin;
+        team_barrier(bar, W * 32);
+        cmin = rb[0];
+#pragma unroll
+        for (int w = 1; w < W; ++w) cmin = fminf(cmin, rb[w * 4]);
+      }
+      if (scan) piv_state = cmin;
+    }
+    if (want_p && safe) piv_state = (S.piv + S.off) + 0.5f * wid;
+    if (!block) off_state = 0.0f;
+  }
+  if (P.state_out && row_ok && lig == 0 && wit == 0 && TK_IN_BOUNDS(row, 1, P.rows, P.status)) {
+    tk_rowstate st;
+    st.pivot = piv_state; st.offset = off_state; st.a = S.a0; st.b = S.b0;
+    P.state_out[row] = st;
+  }
+
+  if (P.out == nullptr) {                      // the row state alone was asked for
+    if (P.status) {
+      if (bad) flags |= TK_FLAG_NONFINITE;
+      if (flags) atomicOr(P.status, flags);
+    }
+    return;
+  }
+
+  // ---- dual map y = rho(clamp(key - tau)), in the order the keys were read.  phi even: a top singleton
+  // is its own minimiser vtop(key) (stationarity rho(key - v) = v), and the sign of theta comes back
+  if constexpr (!MAG) {
+    const float shift = -S.off * inv_lam;
+    if constexpr (WHAT == NT_MASK) {
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        float y[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float a = __saturatef(fmaf(d[4 * c + j], inv_lam, shift));
+          y[j] = Q4 ? a * a * a : a;
+        }
+        io.store(c, y);
+      }
+    } else if constexpr (WHAT == NT_TOPK) {
+      // y theta.  What is read past the row is not stored; a key of -infinity counts as 0
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        float x4[4];
+        io.template load_raw<true>(c, x4);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float a = __saturatef(fmaf(d[4 * c + j], inv_lam, shift));
+          x4[j] = (Q4 ? a * a * a : a) * nt_max_nan(x4[j], -FLT_MAX);
+        }
+        io.store(c, x4);
+        if ((c & 3) == 3) nt_fence();
+      }
+    } else {
+      // The smooth top-k loss and its gradient: sum y (theta - (lambda/p) y^(p-1)) - theta[t] and y - t.  y^(p-1) is the
+      // clamped distance itself.
+      const float lop = (Q4 ? 0.75f : 0.5f) * lam;          // lambda / p
+      const int target = (P.target && row_ok && TK_IN_BOUNDS(row, 1, P.rows, P.status)) ? P.target[row] : -1;
+      const float x_t = (target >= 0 && target < n) ? __ldg(io.src + target) : 0.0f;
+      double acc = 0.0;
+      constexpr int GRP = CH < 4 ? CH : 4;     // chunks whose loads are in flight together
+#pragma unroll
+      for (int c0 = 0; c0 < CH; c0 += GRP) {
+        float x4[GRP][4];
+#pragma unroll
+        for (int c = 0; c < GRP; ++c) io.template load_raw<true>(c0 + c, x4[c]);
+#pragma unroll
+        for (int c = 0; c < GRP; ++c) {
+          float a[4], y[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            a[j] = __saturatef(fmaf(d[4 * (c0 + c) + j], inv_lam, shift));
+            y[j] = Q4 ? a[j] * a[j] * a[j] : a[j];
+          }
+          if (fmaxf(fmaxf(a[0], a[1]), fmaxf(a[2], a[3])) > 0.0f) {       // most of the chunks are 0
+            double t[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              t[j] = (double)y[j] * ((double)(y[j] > 0.0f ? x4[c][j] : 0.0f) - (double)(lop * a[j]));
+            acc += (t[0] + t[1]) + (t[2] + t[3]);
+          }
+          if (target >= 0) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (io.pos(c0 + c) + j == target) y[j] -= 1.0f;
+          }
+          io.store(c0 + c, y);
+        }
+        nt_fence();
+      }
+#pragma unroll
+      for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (W > 1) {
+        double* slot = reinterpret_cast<double*>(red + (phase & 1) * (W * 4));               // (16 bytes per warp)
+        ++phase;
+        if (lane == 0 && TK_IN_BOUNDS(team * (2 * W * 4) + ((phase - 1) & 1) * (W * 4) + wit * 4, 2, TEAMS * 2 * W * 4, P.status)) slot[wit * 2] = acc;
+        team_barrier(bar, W * 32);
+        acc = slot[0];
+#pragma unroll
+        for (int w = 1; w < W; ++w) acc += slot[w * 2];
+      }
+      if (row_ok && lig == 0 && wit == 0 && TK_IN_BOUNDS(row, 1, P.rows, P.status)) {
+        if (target >= 0 && target < n) acc -= (double)x_t;
+        P.loss[row] = (float)acc;
+      }
+    }
+  } else {
+    Math M = make_math(P);
+    M.q4 = Q4; M.mag = true; M.gen = false;
+    const float off = S.off;
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      float x4[4], y[4];
+      io.load(c, x4);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float t = d[4 * c + j] - off;
+        float v = 0.0f;
+        if (t >= wid) v = M.vtop(fabsf(x4[j]));
+        else if (t > 0.0f) v = M.rho(t);
+        y[j] = signbit(x4[j]) ? -v : v;
+      }
+      io.store(c, y);
+      if ((c & 3) == 3) nt_fence();
+    }
+  }
+  if (STAGED) {
+    constexpr int RS = G * E;
+    __syncwarp();
+    const float* tile = smem + warp * (32 * E);
+    const int rows_here = (int)(P.rows - row0 < (long long)R ? P.rows - row0 : (long long)R);
+    float* dst = P.out + row0 * (long long)n;
+    if (n == RS) {
+      const int total = rows_here * n;
+      if (P.vec4) {
+        float4* d4 = reinterpret_cast<float4*>(dst);
+        const float4* t4 = reinterpret_cast<const float4*>(tile);
+        for (int v = lane; 4 * v < total; v += 32)
+          if (TK_IN_BOUNDS(row0 * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(4 * v, 4, 32 * E, P.status)) d4[v] = t4[v];
+      } else {
+        for (int i = lane; i < total; i += 32)
+          if (TK_IN_BOUNDS(row0 * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(i, 1, 32 * E, P.status)) dst[i] = tile[i];
+      }
+    } else {
+      for (int r = 0; r < rows_here; ++r) {
+        if (P.vec4) {
+          float4* d4 = reinterpret_cast<float4*>(dst + (long long)r * n);
+          const float4* t4 = reinterpret_cast<const float4*>(tile + r * RS);
+          for (int v = lane; 4 * v < n; v += 32)
+            if (TK_IN_BOUNDS((row0 + r) * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(r * RS + 4 * v, 4, 32 * E, P.status)) d4[v] = t4[v];
+        } else {
+          for (int i = lane; i < n; i += 32)
+            if (TK_IN_BOUNDS((row0 + r) * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(r * RS + i, 1, 32 * E, P.status)) dst[(long long)r * n + i] = tile[r * RS + i];
+        }
+      }
+    }
+  }
+  if (P.status) {
+    if (bad) flags |= TK_FLAG_NONFINITE;
+    if (flags) atomicOr(P.status, flags);
+  }
+}
+
 // G lanes per row (W == 1) or W warps per row (G == 32), E keys per lane (E / 4 a power of two).
-// KSEL: 0 = moment start, 1 / 2 = k is 1 / 2 (W == 1, phi = x only).  MAG: phi(x) = x^2/2, keys |theta|.
-template <int G, int E, int W, bool Q4, int KSEL, bool STAGED, bool MAG>
+// KSEL: 0 = moment start, 1 / 2 = k is 1 / 2 (W == 1, phi = x only).  WHAT: what is made of the root.  It is a template
+// parameter because the kernel is bound by its registers: with the epilogues in one kernel behind tests, the mask's rows
+// ran slower too (65536 x 1000, p = 4/3: 196 us with topk in the same kernel, 174 alone).
+template <int G, int E, int W, bool Q4, int KSEL, bool STAGED, NtWhat WHAT>
 __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED, G)) tk_newton_kernel(const Problem P, const float zq, const int pf_rows) {
   extern __shared__ float4 nt_smem4[];
+  constexpr bool MAG = WHAT == NT_MAG;
   static_assert(W == 1 || G == 32, "several warps per row: every lane of them belongs to the row");
   static_assert(!STAGED || W == 1, "the staging tile belongs to one warp");
   static_assert(!MAG || KSEL == 0, "the magnitude mode starts from the moments");
@@ -183,41 +450,29 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
   constexpr int TEAMS = BW / W;                      // teams (of W warps) per block
   constexpr int R = W > 1 ? 1 : 32 / G;              // rows per team
   constexpr int CH = E / 4;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int team = warp / W, wit = warp % W;
-  const long long row0 = ((long long)blockIdx.x * TEAMS + team) * R;
+  using Place = NtPlace<G, E, W, STAGED>;
+  float* smem = reinterpret_cast<float*>(nt_smem4);
+  constexpr bool REBUILD = NtRebuild<E, W>::v;
+  const Place at(P, smem, threadIdx.x, blockIdx.x);
+  const int lane = at.lane, warp = at.warp, team = at.team, wit = at.wit, lig = at.lig;
+  const long long row0 = at.row0, row = at.row;
+  const NtIO<G, E, W, STAGED>& io = at.io;
   if (row0 >= P.rows) return;                  // the whole team
   const int n = P.n, k = P.k;
-  const int rl = lane / G, lig = lane % G;
-  const long long row = row0 + rl;
-  const bool row_ok = row < P.rows;
   const float lam = P.lam, inv_lam = P.inv_lam, lam3 = P.lam3;
   float wid = P.lam;                           // phi = x: constant; phi even: follows tau
   constexpr float kTolRel = Q4 ? 1e-7f : 3e-7f;
-  float* smem = reinterpret_cast<float*>(nt_smem4);
   // shared memory: [STAGED: one tile of 32 E floats per warp] [W > 1: two buffers of W * 4 words per team]
   float* red = smem + (STAGED ? BW * 32 * E : 0) + team * (2 * W * 4);
   const int bar = 1 + team;
   int phase = 0;                               // which of the two buffers the next team sum uses
 
-  NtIO<G, E, W, STAGED> io;
-  io.n = n; io.vec4 = P.vec4; io.row_ok = row_ok;
-  io.tl = W > 1 ? wit * 32 + lane : lig;
-  io.rot = nt_rot<E>(lane);
-  // a group past the last row works on the last row again and stores nothing
-  const long long row_c = row_ok ? row : P.rows - 1;
-  io.src = P.theta + row_c * (long long)n;
-  io.dst = P.out + row_c * (long long)n;
-  io.first = row_c * (long long)n; io.extent = P.rows * (long long)n; io.status = P.status;
-  io.lane_in_warp = lane;
-  io.span4 = nullptr;
   if (KSEL != 0) overlap_next();               // k <= 2: no iteration to speak of, the next grid may queue at once
   overlap_wait();
   if (STAGED) {
     // ---- stage the warp's rows (contiguous in memory) in its tile, row stride G * E
     constexpr int RS = G * E;
     float* tile = smem + warp * (32 * E);
-    io.span4 = reinterpret_cast<float4*>(tile + lane * E);
     const int rows_here = (int)(P.rows - row0 < (long long)R ? P.rows - row0 : (long long)R);
     const float* src = P.theta + row0 * (long long)n;
     if (n == RS) {
@@ -403,6 +658,8 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
       nt_step<Q4, MAG>(S, (int)(packed & 0xffffu), (int)(packed >> 16), v[0], Q4 ? v[1] : 0.0f,
                        Q4 ? v[Q4 ? 2 : 0] : 0.0f, k, lam, lam3, wid, tol);
       if (S.repiv) {
+        const Place again = REBUILD ? Place(P, smem, nt_tid(), nt_cta()) : at;
+        const NtIO<G, E, W, STAGED>& io = again.io;
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
           float x4[4];
@@ -415,148 +672,16 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
       }
     }
   }
-  int flags = 0;
-  if (!S.done) {                               // cap reached: keep the last point, say so
-    flags |= TK_FLAG_NOT_CONVERGED;
-    S.a0 = k; S.b0 = k;
-  }
-  if (S.b0 <= S.a0) { S.a0 = k; S.b0 = k; }
-  const bool block = S.b0 > S.a0;
-  if (MAG) wid = nt_width<Q4, true>(S.piv + S.off, lam);   // of the point the last pass classified at
-
-  // ---- row state.  Without a block the VJP classifies by key >= pivot: any value above the
-  // (k+1)-th largest key and not above the k-th serves; tau + lambda/2 is one when lambda is
-  // resolved at the keys' magnitude, else the smallest capped key is looked up.
-  float piv_state = S.piv, off_state = S.off;
-  {
-    const bool want_p = row_ok && !block && !early;
-    const bool safe = wid > 9.6e-7f * (fabsf(S.piv) + fabsf(S.off));
-    const bool scan = want_p && !safe;
-    if (__any_sync(0xffffffffu, scan)) {       // uniform over the warps of a row: they hold the same S
-      float cmin = INFINITY;
-#pragma unroll
-      for (int c = 0; c < CH; ++c) {
-        float x4[4];
-        io.load(c, x4);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (d[4 * c + j] - S.off >= wid) cmin = fminf(cmin, MAG ? fabsf(x4[j]) : x4[j]);
-        if ((c & 3) == 3) nt_fence();
-      }
-      cmin = team_gmin<G>(cmin);
-      if (W > 1) {
-        float* rb = red + (phase & 1) * (W * 4);
-        ++phase;
-        if (lane == 0 && TK_IN_BOUNDS(team * (2 * W * 4) + ((phase - 1) & 1) * (W * 4) + wit * 4, 1, TEAMS * 2 * W * 4, P.status)) rb[wit * 4] = cmin;
-        team_barrier(bar, W * 32);
-        cmin = rb[0];
-#pragma unroll
-        for (int w = 1; w < W; ++w) cmin = fminf(cmin, rb[w * 4]);
-      }
-      if (scan) piv_state = cmin;
-    }
-    if (want_p && safe) piv_state = (S.piv + S.off) + 0.5f * wid;
-    if (!block) off_state = 0.0f;
-  }
-  if (P.state_out && row_ok && lig == 0 && wit == 0 && TK_IN_BOUNDS(row, 1, P.rows, P.status)) {
-    tk_rowstate st;
-    st.pivot = piv_state; st.offset = off_state; st.a = S.a0; st.b = S.b0;
-    P.state_out[row] = st;
-  }
-
-  if (P.out == nullptr) {                      // the row state alone was asked for
-    if (P.status) {
-      if (bad) flags |= TK_FLAG_NONFINITE;
-      if (flags) atomicOr(P.status, flags);
-    }
-    return;
-  }
-
-  // ---- dual map y = rho(clamp(key - tau)), in the order the keys were read.  phi even: a top singleton
-  // is its own minimiser vtop(key) (stationarity rho(key - v) = v), and the sign of theta comes back
-  if (!MAG) {
-    const float shift = -S.off * inv_lam;
-    const bool times_x = P.mode == TK_TOPK;
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-      float y[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float a = __saturatef(fmaf(d[4 * c + j], inv_lam, shift));
-        y[j] = Q4 ? a * a * a : a;
-      }
-      if (times_x) {
-        float x4[4];
-        io.load(c, x4);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) y[j] = (x4[j] == -INFINITY) ? 0.0f : y[j] * x4[j];
-      }
-      io.store(c, y);
-      if (times_x && (c & 3) == 3) nt_fence();
-    }
-  } else {
-    Math M = make_math(P);
-    M.q4 = Q4; M.mag = true; M.gen = false;
-    const float off = S.off;
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-      float x4[4], y[4];
-      io.load(c, x4);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float t = d[4 * c + j] - off;
-        float v = 0.0f;
-        if (t >= wid) v = M.vtop(fabsf(x4[j]));
-        else if (t > 0.0f) v = M.rho(t);
-        y[j] = signbit(x4[j]) ? -v : v;
-      }
-      io.store(c, y);
-      if ((c & 3) == 3) nt_fence();
-    }
-  }
-  if (STAGED) {
-    constexpr int RS = G * E;
-    __syncwarp();
-    const float* tile = smem + warp * (32 * E);
-    const int rows_here = (int)(P.rows - row0 < (long long)R ? P.rows - row0 : (long long)R);
-    float* dst = P.out + row0 * (long long)n;
-    if (n == RS) {
-      const int total = rows_here * n;
-      if (P.vec4) {
-        float4* d4 = reinterpret_cast<float4*>(dst);
-        const float4* t4 = reinterpret_cast<const float4*>(tile);
-        for (int v = lane; 4 * v < total; v += 32)
-          if (TK_IN_BOUNDS(row0 * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(4 * v, 4, 32 * E, P.status)) d4[v] = t4[v];
-      } else {
-        for (int i = lane; i < total; i += 32)
-          if (TK_IN_BOUNDS(row0 * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(i, 1, 32 * E, P.status)) dst[i] = tile[i];
-      }
-    } else {
-      for (int r = 0; r < rows_here; ++r) {
-        if (P.vec4) {
-          float4* d4 = reinterpret_cast<float4*>(dst + (long long)r * n);
-          const float4* t4 = reinterpret_cast<const float4*>(tile + r * RS);
-          for (int v = lane; 4 * v < n; v += 32)
-            if (TK_IN_BOUNDS((row0 + r) * (long long)n + 4 * v, 4, io.extent, P.status) && TK_IN_BOUNDS(r * RS + 4 * v, 4, 32 * E, P.status)) d4[v] = t4[v];
-        } else {
-          for (int i = lane; i < n; i += 32)
-            if (TK_IN_BOUNDS((row0 + r) * (long long)n + i, 1, io.extent, P.status) && TK_IN_BOUNDS(r * RS + i, 1, 32 * E, P.status)) dst[(long long)r * n + i] = tile[r * RS + i];
-        }
-      }
-    }
-  }
-  if (P.status) {
-    if (bad) flags |= TK_FLAG_NONFINITE;
-    if (flags) atomicOr(P.status, flags);
-  }
+  const Place fin = REBUILD ? Place(P, smem, nt_tid(), nt_cta()) : at;
+  nt_finish<G, E, W, Q4, STAGED, WHAT>(P, fin, S, d, wid, early, bad, phase, smem);
 }
 
-template <int G, int E, int W, bool Q4, int KSEL, bool STAGED, bool MAG>
+template <int G, int E, int W, bool Q4, int KSEL, bool STAGED, NtWhat WHAT>
 cudaError_t nt_launch(const Problem& P, float zq, cudaStream_t stream) {
   constexpr int BW = kNtWarps > W ? kNtWarps : W;
   constexpr int TEAMS = BW / W;
   constexpr int smem = (STAGED ? BW * 32 * E * (int)sizeof(float) : 0) + (W > 1 ? TEAMS * 2 * W * 4 * (int)sizeof(float) : 0);
-  auto kern = tk_newton_kernel<G, E, W, Q4, KSEL, STAGED, MAG>;
+  auto kern = tk_newton_kernel<G, E, W, Q4, KSEL, STAGED, WHAT>;
   if (smem > 48 * 1024) {
     static bool configured[64];
     int dev = 0;
@@ -577,20 +702,24 @@ cudaError_t nt_launch(const Problem& P, float zq, cudaStream_t stream) {
 }
 
 // KS: the shape also has the variants that track the k + 1 largest keys (k <= 2, phi = x)
+template <int G, int E, int W, bool KS, bool STAGED, NtWhat WHAT>
+cudaError_t nt_launch_k(const Problem& P, float zq, cudaStream_t stream) {
+  const bool q4 = P.q4 != 0;
+  if (KS && P.k == 1)
+    return q4 ? nt_launch<G, E, W, true, KS ? 1 : 0, STAGED, WHAT>(P, zq, stream)
+              : nt_launch<G, E, W, false, KS ? 1 : 0, STAGED, WHAT>(P, zq, stream);
+  if (KS && P.k == 2)
+    return q4 ? nt_launch<G, E, W, true, KS ? 2 : 0, STAGED, WHAT>(P, zq, stream)
+              : nt_launch<G, E, W, false, KS ? 2 : 0, STAGED, WHAT>(P, zq, stream);
+  return q4 ? nt_launch<G, E, W, true, 0, STAGED, WHAT>(P, zq, stream)
+            : nt_launch<G, E, W, false, 0, STAGED, WHAT>(P, zq, stream);
+}
+
 template <int G, int E, int W, bool KS, bool STAGED>
 cudaError_t nt_launch_q(const Problem& P, float zq, cudaStream_t stream) {
-  const bool q4 = P.q4 != 0;
-  if (P.mode == TK_TOPKMAG)
-    return q4 ? nt_launch<G, E, W, true, 0, STAGED, true>(P, zq, stream)
-              : nt_launch<G, E, W, false, 0, STAGED, true>(P, zq, stream);
-  if (KS && P.k == 1)
-    return q4 ? nt_launch<G, E, W, true, KS ? 1 : 0, STAGED, false>(P, zq, stream)
-              : nt_launch<G, E, W, false, KS ? 1 : 0, STAGED, false>(P, zq, stream);
-  if (KS && P.k == 2)
-    return q4 ? nt_launch<G, E, W, true, KS ? 2 : 0, STAGED, false>(P, zq, stream)
-              : nt_launch<G, E, W, false, KS ? 2 : 0, STAGED, false>(P, zq, stream);
-  return q4 ? nt_launch<G, E, W, true, 0, STAGED, false>(P, zq, stream)
-            : nt_launch<G, E, W, false, 0, STAGED, false>(P, zq, stream);
+  if (P.mode == TK_TOPKMAG) return nt_launch_k<G, E, W, false, STAGED, NT_MAG>(P, zq, stream);
+  if (P.mode == TK_TOPK) return nt_launch_k<G, E, W, KS, STAGED, NT_TOPK>(P, zq, stream);
+  return P.loss ? nt_launch_k<G, E, W, KS, STAGED, NT_LOSS>(P, zq, stream) : nt_launch_k<G, E, W, KS, STAGED, NT_MASK>(P, zq, stream);
 }
 
 }  // namespace

@@ -1190,3 +1190,35 @@ def test_long_rows_over_the_grid(n, kind):
         # (the gradient jumps where an element enters the pooled block: elements within 1e-5 of its edge are left out)
         o, e = out.cpu().numpy().astype(np.float64), rel_err(grad.cpu().numpy(), tko.vjp(x, g, k, p, lam, mode))
         assert (e > TOL).sum() <= 2, (kind, mode, p, int((e > TOL).sum()), e.max())
+
+
+@pytest.mark.parametrize("p", [2.0, P43])
+@pytest.mark.parametrize("n", [8, 9, 16, 17, 33, 64, 65, 128, 129, 257, 512, 515, 1024, 1025, 2049, 4097, 8193, 16385, 32768])
+def test_loss_and_topk_values_at_team_edges(n, p):
+    """The loss made by the forward kernel itself and the topk values, at the edges of every row layout: targets on the
+    first and the last key, none, outside the row; k tracked exactly (1, 2) and from the moments."""
+    from oracle import tko
+    from parity import rel_err, TOL
+    rows = 37 if n < 4096 else 3
+    x = rows_of(n, rows, 13000 + n, 2.0)
+    tgt = np.random.default_rng(n).integers(0, n, size=rows).astype(np.int32)
+    tgt[0], tgt[1], tgt[2] = n - 1, 0, -1
+    if rows > 3:
+        tgt[3] = n
+    th, tg = torch.from_numpy(x).cuda(), torch.from_numpy(tgt).cuda()
+    for k in sorted({1, 2, 5, n // 2, n}):
+        loss, grad, out = torch.full((rows,), float("nan"), device="cuda"), torch.full_like(th, float("nan")), torch.empty_like(th)
+        again, state = torch.empty_like(th), tk.new_state(rows)
+        tk.tk_topk_loss(th, tg, rows, n, k, p, 0.5, loss, grad, state_out=state)
+        tk.tk_fwd(th, rows, n, k, p, 0.5, tk.TK_TOPK, out)
+        tk.tk_fwd(th, rows, n, k, p, 0.5, tk.TK_MASK, again)
+        torch.cuda.synchronize()
+        lref, gref = tko.topk_loss(x, tgt, k, p, 0.5)
+        assert rel_err(loss.cpu().numpy(), lref).max() <= TOL, k
+        assert rel_err(grad.cpu().numpy(), gref).max() <= TOL, k
+        assert rel_err(out.cpu().numpy(), tko.fwd(x, k, p, 0.5, tk.TK_TOPK)).max() <= TOL, k
+        hot = torch.zeros_like(th)
+        for r in range(rows):
+            if 0 <= tgt[r] < n:
+                hot[r, int(tgt[r])] = 1.0
+        assert torch.equal(grad, again - hot), k          # the same mask, bit for bit
