@@ -39,31 +39,22 @@ constexpr int vt_min_blocks(int E, int W, int MODE) {
   return team_min_blocks(E >= 32 ? 16 : (MODE == TK_MASK ? 32 : 24), W);
 }
 
-// The sums of a row shared by the CL thread blocks of a cluster: each block leaves its own total in its
-// shared memory, a cluster barrier, then every block adds the CL totals in rank order (same order, same
-// result in every block).
-template <int NV, int CL>
-__device__ __forceinline__ void vt_cluster_sum(float (&v)[NV], float* slot, cg::cluster_group& cluster) {
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) slot[i] = v[i];
-  }
+// A value of every thread block of the row's cluster to every other: thread r of a block writes its block's value into block
+// r's shared memory, and after one cluster barrier each block reads its own.  No block touches another's memory after the
+// barrier, so none has to stay for the others.  An SM holds two blocks, so little
+// hides a barrier over four: 2048 x 32768, mask, p = 2: 187 us with three of them per row (each block's sum read by the others,
+// twice, and a last one to leave), 163 with one; topk 354 -> 338, phi even (two) 404 -> 401.
+template <int CL>
+__device__ __forceinline__ void vt_cluster_share(float4 mine, float4* slots, unsigned crank, cg::cluster_group& cluster) {
+  if (threadIdx.x < CL) cluster.map_shared_rank(slots, threadIdx.x)[crank] = mine;
   cluster.sync();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = 0.0f;
-#pragma unroll
-  for (int r = 0; r < CL; ++r) {
-    const float* peer = cluster.map_shared_rank(slot, (unsigned)r);
-#pragma unroll
-    for (int i = 0; i < NV; ++i) v[i] += peer[i];
-  }
 }
 
 // QM: 0 = q is 2, 1 = q is 4, 2 = any other q (rho' through powf).  MODE: tk_mode.  CL: thread blocks
 // per row (above 1: a cluster of CL blocks, each with its share of the row in its registers).
 template <int G, int E, int W, int QM, int MODE, int CL>
 __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk_vjp_team_kernel(const Problem P) {
-  extern __shared__ float vt_smem[];
+  extern __shared__ __align__(16) float vt_smem[];
   static_assert(W == 1 || G == 32, "several warps per row: every lane of them belongs to the row");
   static_assert(CL == 1 || W >= kTeamWarps, "a cluster shares one row: one team per block");
   constexpr int BW = kTeamWarps > W ? kTeamWarps : W;
@@ -92,6 +83,8 @@ __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk
   const float* g_row = P.gout + row_c * (long long)n;
   float* o_row = P.out + row_c * (long long)n;
 
+  // every block of the cluster has to run before another writes into its shared memory: waited for after the loads
+  if (CL > 1) cluster.barrier_arrive();
   overlap_wait();
   // ---- theta and g: every load is unconditional (a chunk past the row re-reads its start)
   float x[E], g[E];
@@ -153,15 +146,25 @@ __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk
     AD[1] += dr;
   }
   overlap_next();
+  if (CL > 1) cluster.barrier_wait();
   float ratio = 0.0f, delta = 0.0f;
   if (__any_sync(0xffffffffu, has_block)) {    // the warps of a row agree: same row state
     uint32_t none = 0;
     team_allsum<G, W, 2>(AD, none, red, wit, lane, bar);
-    float* xch = vt_smem + TEAMS * (2 * W * 4);              // CL == 2: two slots of four words
-    if (CL > 1) vt_cluster_sum<2, CL>(AD, xch, cluster);
+    float4* xch = reinterpret_cast<float4*>(vt_smem + TEAMS * (2 * W * 4));    // CL > 1: two times CL slots
+    // With phi = x the blocks of a cluster sum the residuals about their own means and then exchange once: the mean of the
+    // row is the mean of theirs weighted by D, and what is rounded away in D counts by their distance only.  With phi even
+    // fm weighs in as a mean of 0, at any distance: the row's mean is exchanged first there.
+    constexpr bool TWO = CL > 1 && MAG;
+    if (TWO) {
+      vt_cluster_share<CL>(make_float4(AD[0], AD[1], 0.0f, 0.0f), xch, crank, cluster);
+      AD[0] = AD[1] = 0.0f;
+#pragma unroll
+      for (int r = 0; r < CL; ++r) { AD[0] += xch[r].x; AD[1] += xch[r].y; }
+    }
     float D = AD[1];
     if (MAG) D += fm;
-    const bool ok = has_block && D > 0.0f;
+    bool ok = has_block && D > 0.0f;
     ratio = ok ? AD[0] / D : 0.0f;
     float A2[1] = {0.f};
 #pragma unroll
@@ -172,12 +175,29 @@ __global__ void __launch_bounds__(team_threads(W), vt_min_blocks(E, W, MODE)) tk
       A2[0] = fmaf(fabsf(w[i]), fmaf(chi, g[i], -ratio), A2[0]);   // |w| = rho'
     }
     team_allsum<G, W, 1>(A2, none, red + W * 4, wit, lane, bar);
-    if (CL > 1) {
-      vt_cluster_sum<1, CL>(A2, xch + 4, cluster);
-      cluster.sync();                          // no block leaves while the other may still read its slot
+    if (TWO) {
+      vt_cluster_share<CL>(make_float4(A2[0], 0.0f, 0.0f, 0.0f), xch + CL, crank, cluster);
+      A2[0] = 0.0f;
+#pragma unroll
+      for (int r = 0; r < CL; ++r) A2[0] += xch[CL + r].x;
     }
-    if (MAG) A2[0] -= fm * ratio;
-    delta = ok ? A2[0] / D : 0.0f;
+    if (CL > 1 && !TWO) {
+      vt_cluster_share<CL>(make_float4(D, ratio, A2[0], 0.0f), xch, crank, cluster);
+      double num = 0.0, den = 0.0;
+#pragma unroll
+      for (int r = 0; r < CL; ++r) {
+        const float4 v = xch[r];
+        num += (double)v.x * (double)v.y + (double)v.z;
+        den += (double)v.x;
+      }
+      ok = has_block && den > 0.0;
+      const double mean = ok ? num / den : 0.0;
+      ratio = (float)mean;
+      delta = (float)(mean - (double)ratio);
+    } else {
+      if (MAG) A2[0] -= fm * ratio;
+      delta = ok ? A2[0] / D : 0.0f;
+    }
   }
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
@@ -206,7 +226,7 @@ template <int G, int E, int W, int QM, int MODE, int CL>
 cudaError_t vt_launch(const Problem& P, cudaStream_t stream) {
   constexpr int BW = kTeamWarps > W ? kTeamWarps : W;
   constexpr int TEAMS = BW / W;
-  constexpr int smem = (TEAMS * 2 * W * 4 + (CL > 1 ? 8 : 0)) * (int)sizeof(float);
+  constexpr int smem = (TEAMS * 2 * W * 4 + (CL > 1 ? 8 * CL : 0)) * (int)sizeof(float);
   constexpr long long rows_per_block = (long long)TEAMS * (W > 1 ? 1 : 32 / G);
   if (CL == 1) {
     const unsigned blocks = (unsigned)((P.rows + rows_per_block - 1) / rows_per_block);

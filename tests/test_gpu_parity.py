@@ -1222,3 +1222,17 @@ def test_loss_and_topk_values_at_team_edges(n, p):
             if 0 <= tgt[r] < n:
                 hot[r, int(tgt[r])] = 1.0
         assert torch.equal(grad, again - hot), k          # the same mask, bit for bit
+
+
+@pytest.mark.parametrize("mode", [tk.TK_MASK, tk.TK_TOPK, tk.TK_TOPKMAG])
+@pytest.mark.parametrize("n", [16385, 16388, 24577, 32767, 32768])
+def test_vjp_of_rows_shared_by_a_cluster(n, mode):
+    """Rows of four thread blocks: blocks without a member of the pooled block, a block that sits in one of them
+    whole, none at all; with the exchange made once (phi = x) and twice (phi even)."""
+    from parity import run_case
+    for p in (2.0, P43):
+        for k, lam in [(n // 8, 1.0), (3, 0.5), (n - 1, 0.1), (n, 1.0)]:
+            x = rows_of(n, 5, 14000 + n + mode)
+            x[1] = np.sort(x[1])                   # the pooled block next to each other
+            x[2] = np.sort(x[2])[::-1]
+            run_case(x, k, p, lam, mode, wl.cotangent_like(x, n), label=f"n={n} k={k} lam={lam} mode={mode} p={p}")
