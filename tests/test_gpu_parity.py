@@ -1236,3 +1236,15 @@ def test_vjp_of_rows_shared_by_a_cluster(n, mode):
             x[1] = np.sort(x[1])                   # the pooled block next to each other
             x[2] = np.sort(x[2])[::-1]
             run_case(x, k, p, lam, mode, wl.cotangent_like(x, n), label=f"n={n} k={k} lam={lam} mode={mode} p={p}")
+
+
+@pytest.mark.parametrize("p", [2.0, P43])
+@pytest.mark.parametrize("n,k,lam", [(400, 8, 0.1), (1000, 8, 0.1), (1000, 5, 0.5), (3000, 10, 0.02)])
+def test_last_step_below_the_resolution_of_the_threshold(n, k, lam, p):
+    """Class logits with ties and a small lambda: a pair of keys carries the block, and the last step of the
+    iteration is often smaller than one unit in the last place of the offset it is added to."""
+    from parity import run_case
+    for scale in (3.0, 30.0):
+        x = rows_of(n, 500, 15000 + n, scale)
+        x[:, : n // 10] = x[:, n // 2: n // 2 + n // 10]
+        run_case(x, k, p, lam, tk.TK_MASK, wl.cotangent_like(x, n), label=f"n={n} k={k} lam={lam} p={p} scale={scale}")
