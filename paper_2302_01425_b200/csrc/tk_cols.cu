@@ -164,7 +164,6 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
   constexpr float kTolRel = Q4 ? 1e-7f : 3e-7f;
   int phase = 0;
 
-  overlap_next();
   overlap_wait();
   float d[E];
   col_each<E>(R, [&](int i, auto fast) { d[i] = X.template load<decltype(fast)::value>(i, R); });
@@ -365,7 +364,6 @@ __global__ void __maxnreg__(E <= 16 ? (MODE == TK_MASK ? 56 : 64) : 112) tk_cols
   const ColRows<Off> R(n);
   const ColMatrix<Off> X(A.theta, A.ld_theta, col0, c, R, cols, P.status);
   const ColMatrix<Off> GM(A.gout, A.ld_gout, col0, c, R, cols, P.status);
-  overlap_next();
   overlap_wait();
   float x[E], g[E];
   col_each<E>(R, [&](int i, auto fast) {

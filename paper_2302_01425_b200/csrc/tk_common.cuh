@@ -89,6 +89,9 @@ inline int sm_count() {
 // After the row has been read and the starting guess is known was the best place for the Newton kernel and its VJP
 // (forward + VJP, us: at the kernel's start / there: 10007 x 60 p = 4/3 14.0 / 12.4, 16384 x 32 k = 4 22.1 / 13.6,
 // 4000 x 200 17.4 / 12.6, 4096 x 512 17.6 / 16.0; 16384 x 64 k = 2 7.3 / 7.6); rows in whole waves do not care.
+// The kernels whose blocks work long on few loads (general w, permutations, sweeps, columns, sorted rows) do not call it: the
+// next grid may start when their blocks have ended.  With it at their start, steps of a few blocks queued back to back
+// put the waiting blocks of several grids on the same few SMs (one such step: 42 us alone, 236 in a row).
 __device__ __forceinline__ void overlap_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -31,7 +31,6 @@ __global__ void __launch_bounds__(256) tk_loss_kernel(const float* theta,
   const int lane = threadIdx.x % TPR;
   const long long row = (long long)blockIdx.x * RPB + threadIdx.x / TPR;
   const bool live = row < rows;
-  overlap_next();
   overlap_wait();
   double acc = 0.0;
   const float* x = theta + (live ? row : 0) * (long long)n;

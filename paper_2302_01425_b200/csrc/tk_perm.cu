@@ -45,7 +45,6 @@ __global__ void __launch_bounds__(RankGeom<G, W>::THREADS, (W == 1 ? 6 : (W >= 1
   int* work = reinterpret_cast<int*>(sm + R * NP);
   const bool mag = P.mode == TK_TOPKMAG;
 
-  overlap_next();
   overlap_wait();
   float x[E], r[E];
   bool bad = false;

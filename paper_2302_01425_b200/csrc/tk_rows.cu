@@ -336,7 +336,6 @@ __global__ void __launch_bounds__(kRowsThreads, E <= 16 ? 6 : 3) tk_rows_kernel(
   int flags = 0;
 
   // elements 4 h .. 4 h + 3 of the lane's E consecutive elements of a row (zeros past the row's end)
-  overlap_next();
   overlap_wait();
   auto load4 = [&](const float* base, bool live, int h, float (&v4)[4]) {
     const int e0 = E * lig + 4 * h;

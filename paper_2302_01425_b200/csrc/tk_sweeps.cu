@@ -209,7 +209,6 @@ __global__ void __launch_bounds__(RankGeom<G, W>::THREADS, (W == 1 ? 5 : (W >= 1
   float* ys = work + rl * 2 * SwGeom<G, W>::VN;
   const float* x_row = P.theta + first;
 
-  overlap_next();
   overlap_wait();
   float key[E], r[E];
   bool bad = false;

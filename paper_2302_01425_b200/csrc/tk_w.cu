@@ -176,7 +176,6 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
   const uint32_t magic = n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u;
   auto row_of = [&](int e) -> int { return R == 1 ? 0 : (n > 1 ? (int)__umulhi((uint32_t)e, magic) : e); };
 
-  overlap_next();
   overlap_wait();
   // ---- theta as it lies in memory, w by rank (in the keys' array, which is free until the sort is done).  Every
   // load is unconditional (past the end the last element again), so the loads of a lane are all in flight at once
