@@ -38,11 +38,12 @@ cudaError_t launch_hard(const float* theta, const int32_t* perm, float* out, lon
                         int mode, cudaStream_t stream);
 // [n, cols] with leading dimension <-> contiguous [cols, n] (tk_transpose.cu)
 cudaError_t launch_transpose(const float* in, long long in_rows, long long in_cols, long long in_ld, float* out,
-                             long long out_ld, cudaStream_t stream);
+                             long long out_ld, float* copy, cudaStream_t stream);
 // the operator along the slow axis without a transpose (tk_cols.cu)
 int cols_direct_max_n();
 cudaError_t launch_cols_fwd(const Problem& P, long long ld_theta, long long ld_out, float* copy, cudaStream_t stream);
-cudaError_t launch_cols_vjp(const Problem& P, long long ld_theta, long long ld_gout, long long ld_out, cudaStream_t stream);
+cudaError_t launch_cols_vjp(const Problem& P, long long ld_theta, long long ld_gout, long long ld_out, float* copy,
+                            cudaStream_t stream);
 // relaxed operator over the permutahedron of any sorted w (tk_w.cu)
 int w_max_n();
 cudaError_t launch_w(const Problem& P, const float* w, long long w_rows, cudaStream_t stream);
@@ -416,10 +417,11 @@ tk_status tk_topk_loss(const float* theta, const int32_t* target, int64_t rows, 
 }
 
 // ---- the operator along the slow axis.  p = 2 and p = 4/3, columns of up to cols_direct_max_n() rows: kernels that work
-// on the matrix as it lies in memory, forward pass by the threshold form and VJP from saved state.  Everything else (a
-// permutation, a solver that sorts, general p, a VJP without saved state, longer columns): transpose into the workspace,
-// row kernels, transpose back.  The workspace's first slab keeps a copy of theta for a VJP without theta: as [n, cols]
-// where the direct kernels serve this shape (whatever the forward pass itself used), transposed elsewhere.
+// on the matrix as it lies in memory, forward pass by the threshold form and VJP from row state (without a saved one the
+// forward kernel runs again for it alone).  Everything else (a permutation, a solver that sorts, general p, longer
+// columns): transpose into the workspace, row kernels, transpose back.  Every call that is given theta leaves a copy of
+// it in the workspace's first slab, for a VJP without theta: as [n, cols] where the direct kernels serve this shape
+// (whatever the call itself used), transposed elsewhere.  Nothing else is ever written there.
 static bool cols_direct(int64_t n, double qm1) { return qm1 == 0.0 && n <= tk::cols_direct_max_n(); }
 
 static size_t cols_slab_bytes(int64_t n, int64_t cols) {
@@ -461,19 +463,15 @@ tk_status tk_fwd_cols(const float* theta, int64_t n, int64_t cols, int64_t ld, i
     P.what = tk::W_FWD;
     P.state_out = opts->state_out;
     P.status = opts->status_out;
-    return tk::launch_cols_fwd(P, ld, ld, opts->state_out ? slab[0] : nullptr, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return tk::launch_cols_fwd(P, ld, ld, slab[0], st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
   }
   float* theta_t = slab[direct ? 2 : 0];
-  if (tk::launch_transpose(theta, n, cols, ld, theta_t, n, st) != cudaSuccess) return TK_ERR_CUDA;
+  if (tk::launch_transpose(theta, n, cols, ld, theta_t, n, direct ? slab[0] : nullptr, st) != cudaSuccess) return TK_ERR_CUDA;
   tk_opts inner = *opts;
   inner.workspace = nullptr; inner.workspace_bytes = 0;
   s = tk_fwd_ex(theta_t, cols, n, k, p, lambda, mode, slab[1], &inner, stream);
   if (s != TK_OK) return s;
-  if (direct && opts->state_out &&
-      cudaMemcpy2DAsync(slab[0], (size_t)cols * sizeof(float), theta, (size_t)ld * sizeof(float), (size_t)cols * sizeof(float),
-                        (size_t)n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return TK_ERR_CUDA;
-  return tk::launch_transpose(slab[1], cols, n, n, out, ld, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return tk::launch_transpose(slab[1], cols, n, n, out, ld, nullptr, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
 }
 
 tk_status tk_vjp_cols(const float* theta, const float* grad_out, int64_t n, int64_t cols, int64_t ld,
@@ -482,7 +480,7 @@ tk_status tk_vjp_cols(const float* theta, const float* grad_out, int64_t n, int6
   float* slab[3] = {nullptr, nullptr, nullptr};
   tk_status s = check_cols(n, cols, ld, opts, slab);
   if (s != TK_OK) return s;
-  // theta == NULL: the transposed copy a forward call left in the workspace (needs its row state too)
+  // theta == NULL: the copy that the last call with theta left in the workspace (needs its row state too)
   const bool reuse = theta == nullptr && opts && opts->state_out != nullptr;
   int q4 = 0; double qm1 = 0.0;
   s = check_common(reuse ? (const void*)slab : (const void*)theta, cols, n, k, p, lambda, mode, &q4, &qm1);
@@ -490,23 +488,32 @@ tk_status tk_vjp_cols(const float* theta, const float* grad_out, int64_t n, int6
   if (cols == 0) return TK_OK;
   if (grad_out == nullptr || grad_theta == nullptr) return TK_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  if (cols_direct(n, qm1) && opts->state_out) {
+  // (a single row is its own transpose: the copy is right either way, and two slabs of it do not hold the row state)
+  if (cols_direct(n, qm1) && (opts->state_out || n > 1)) {
     tk::Problem P;
     fill(P, reuse ? slab[0] : theta, cols, n, k, q4, qm1, lambda, mode);
+    P.status = opts->status_out;
+    P.state_in = opts->state_out;
+    if (!P.state_in) {                          // no saved state: the forward kernel again, its row state in the other slabs
+      tk::Problem F = P;
+      F.what = tk::W_FWD;
+      F.state_out = reinterpret_cast<tk_rowstate*>(slab[1]);
+      if (tk::launch_cols_fwd(F, ld, ld, slab[0], st) != cudaSuccess) return TK_ERR_CUDA;
+      P.state_in = F.state_out;
+    }
     P.gout = grad_out;
     P.out = grad_theta;
     P.what = tk::W_VJP;
-    P.state_in = opts->state_out;
-    P.status = opts->status_out;
-    return tk::launch_cols_vjp(P, reuse ? cols : ld, ld, ld, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return tk::launch_cols_vjp(P, reuse ? cols : ld, ld, ld, reuse || !opts->state_out ? nullptr : slab[0], st) == cudaSuccess
+               ? TK_OK : TK_ERR_CUDA;
   }
-  if (!reuse && tk::launch_transpose(theta, n, cols, ld, slab[0], n, st) != cudaSuccess) return TK_ERR_CUDA;
-  if (tk::launch_transpose(grad_out, n, cols, ld, slab[1], n, st) != cudaSuccess) return TK_ERR_CUDA;
+  if (!reuse && tk::launch_transpose(theta, n, cols, ld, slab[0], n, nullptr, st) != cudaSuccess) return TK_ERR_CUDA;
+  if (tk::launch_transpose(grad_out, n, cols, ld, slab[1], n, nullptr, st) != cudaSuccess) return TK_ERR_CUDA;
   tk_opts inner = *opts;
   inner.workspace = nullptr; inner.workspace_bytes = 0;
   s = tk_vjp(slab[0], slab[1], cols, n, k, p, lambda, mode, slab[2], &inner, stream);
   if (s != TK_OK) return s;
-  return tk::launch_transpose(slab[2], cols, n, n, grad_theta, ld, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return tk::launch_transpose(slab[2], cols, n, n, grad_theta, ld, nullptr, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
 }
 
 // ---- any sorted w: relaxed linear maximisation over the permutahedron P(w)

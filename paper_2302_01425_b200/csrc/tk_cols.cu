@@ -34,7 +34,7 @@ struct ColArgs {
   const float* theta; long long ld_theta;      // [n, cols]
   const float* gout; long long ld_gout;        // VJP
   float* out; long long ld_out;
-  float* copy;                                 // forward: contiguous [n, cols] copy of theta for a later VJP, or null
+  float* copy;                                 // contiguous [n, cols] copy of theta for a later VJP, or null
 };
 
 // One slot of a column's sums: 2 or 4 words, moved as a vector.
@@ -315,6 +315,11 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
     st.pivot = piv_state; st.offset = off_state; st.a = T.a0; st.b = T.b0;
     P.state_out[col] = st;
   }
+  if (P.status) {
+    if (bad) flags |= TK_FLAG_NONFINITE;
+    if (flags) atomicOr(P.status, flags);
+  }
+  if (P.out == nullptr) return;                // the row state alone was asked for (a VJP without one)
 
   // ---- dual map
   const ColRows<Off> Ro = R.again();
@@ -344,10 +349,6 @@ __global__ void __maxnreg__(E <= 16 ? 64 : 80) tk_cols_fwd_kernel(const Problem 
       if ((i & 3) == 3) asm volatile("" ::: "memory");
     });
   }
-  if (P.status) {
-    if (bad) flags |= TK_FLAG_NONFINITE;
-    if (flags) atomicOr(P.status, flags);
-  }
 }
 
 // VJP from saved row state (the sums and formulas of tk_vjp_team.cu), theta and the cotangent in registers.  The mask
@@ -370,6 +371,11 @@ __global__ void __maxnreg__(E <= 16 ? (MODE == TK_MASK ? 56 : 64) : 112) tk_cols
     x[i] = X.template load<decltype(fast)::value>(i, R);
     g[i] = GM.template load<decltype(fast)::value>(i, R);
   });
+  if (A.copy) {
+    const ColRows<Off> Rc = R.again();
+    const ColMatrix<Off> C(A.copy, cols, col0, c, Rc, cols, P.status);
+    col_each<E>(Rc, [&](int i, auto fast) { C.template store<decltype(fast)::value>(i, Rc, col_ok, x[i]); });
+  }
   const tk_rowstate st = P.state_in[col0 + c];
   const bool has_block = st.b > st.a;
   const float piv = st.pivot, off = st.offset;
@@ -485,7 +491,8 @@ inline bool col_small(int n, long long ld) { return (long long)n * ld < (1ll << 
 // Longest column these kernels hold: 16 warps of 32 rows per lane.
 int cols_direct_max_n() { return kColSlices * kColMaxWarps * 32; }
 
-// Forward pass (p = 2 or 4/3, no permutation output) on column-strided data; P.rows = number of columns.
+// Forward pass (p = 2 or 4/3, no permutation output) on column-strided data; P.rows = number of columns.  P.out may be null:
+// the row state alone.
 cudaError_t launch_cols_fwd(const Problem& P, long long ld_theta, long long ld_out, float* copy, cudaStream_t stream) {
   ColArgs A = {};
   A.theta = P.theta; A.ld_theta = ld_theta; A.out = P.out; A.ld_out = ld_out; A.copy = copy;
@@ -497,9 +504,11 @@ cudaError_t launch_cols_fwd(const Problem& P, long long ld_theta, long long ld_o
 }
 
 // VJP from saved row state on column-strided data.
-cudaError_t launch_cols_vjp(const Problem& P, long long ld_theta, long long ld_gout, long long ld_out, cudaStream_t stream) {
+cudaError_t launch_cols_vjp(const Problem& P, long long ld_theta, long long ld_gout, long long ld_out, float* copy,
+                            cudaStream_t stream) {
   ColArgs A = {};
   A.theta = P.theta; A.ld_theta = ld_theta; A.gout = P.gout; A.ld_gout = ld_gout; A.out = P.out; A.ld_out = ld_out;
+  A.copy = copy;
   const bool small = col_small(P.n, ld_theta) && col_small(P.n, ld_gout) && col_small(P.n, ld_out);
   if (P.n <= kColSlices * kColMaxWarps * 16) return small ? cols_vjp<16, uint32_t>(P, A, stream) : cols_vjp<16, uint64_t>(P, A, stream);
   return small ? cols_vjp<32, uint32_t>(P, A, stream) : cols_vjp<32, uint64_t>(P, A, stream);

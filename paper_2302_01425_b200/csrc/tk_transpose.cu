@@ -8,10 +8,12 @@ namespace tk {
 
 namespace {
 
-// out[c * out_ld + r] = in[r * in_ld + c] for r < in_rows, c < in_cols
+// out[c * out_ld + r] = in[r * in_ld + c] for r < in_rows, c < in_cols; copy (may be null): the same [in_rows, in_cols]
+// matrix without the gaps of its leading dimension
 __global__ void __launch_bounds__(256) tk_transpose_kernel(const float* __restrict__ in, long long in_rows,
                                                            long long in_cols, long long in_ld,
-                                                           float* __restrict__ out, long long out_ld) {
+                                                           float* __restrict__ out, long long out_ld,
+                                                           float* __restrict__ copy) {
   __shared__ float tile[32][33];
   // tiles are numbered along a 1-D grid (either side of the matrix can exceed the 65535 blocks of gridDim.y)
   const long long tiles_c = (in_cols + 31) / 32;
@@ -20,7 +22,11 @@ __global__ void __launch_bounds__(256) tk_transpose_kernel(const float* __restri
 #pragma unroll
   for (int j = 0; j < 32; j += 8) {
     const long long r = r0 + ty + j, c = c0 + tx;
-    if (r < in_rows && c < in_cols) tile[ty + j][tx] = __ldg(in + r * in_ld + c);
+    if (r < in_rows && c < in_cols) {
+      const float v = __ldg(in + r * in_ld + c);
+      tile[ty + j][tx] = v;
+      if (copy) copy[r * in_cols + c] = v;
+    }
   }
   __syncthreads();
 #pragma unroll
@@ -33,10 +39,10 @@ __global__ void __launch_bounds__(256) tk_transpose_kernel(const float* __restri
 }  // namespace
 
 cudaError_t launch_transpose(const float* in, long long in_rows, long long in_cols, long long in_ld, float* out,
-                             long long out_ld, cudaStream_t stream) {
+                             long long out_ld, float* copy, cudaStream_t stream) {
   const long long tiles = ((in_cols + 31) / 32) * ((in_rows + 31) / 32);
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-  tk_transpose_kernel<<<(unsigned)tiles, 256, 0, stream>>>(in, in_rows, in_cols, in_ld, out, out_ld);
+  tk_transpose_kernel<<<(unsigned)tiles, 256, 0, stream>>>(in, in_rows, in_cols, in_ld, out, out_ld, copy);
   return cudaGetLastError();
 }
 

@@ -1248,3 +1248,51 @@ def test_last_step_below_the_resolution_of_the_threshold(n, k, lam, p):
         x = rows_of(n, 500, 15000 + n, scale)
         x[:, : n // 10] = x[:, n // 2: n // 2 + n // 10]
         run_case(x, k, p, lam, tk.TK_MASK, wl.cotangent_like(x, n), label=f"n={n} k={k} lam={lam} p={p} scale={scale}")
+
+
+@pytest.mark.parametrize("p,mode", [(2.0, tk.TK_MASK), (P43, tk.TK_TOPKMAG)])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 64, 65, 400, 2048, 2049])
+def test_slow_axis_vjp_without_theta_reads_the_last_theta_given(n, p, mode):
+    """tk_vjp_cols without theta after every kind of call that leaves theta in the workspace: a forward pass with and without
+    saved state, a VJP with theta that solves again (which must not disturb the copy's layout), a VJP with theta and
+    state on a workspace no forward pass has seen."""
+    from oracle import tko
+    from parity import rel_err, TOL
+    cols, k, lam = 11, max(1, n // 5), 0.7
+    ld = cols + 2
+    (x, x2), g = (rows_of(n, ld, 16000 + n + i, 1.0).T.copy() for i in (0, 1)), rows_of(n, ld, 16500 + n, 1.0).T.copy()
+    th, th2, gt = (torch.from_numpy(a).cuda() for a in (x, x2, g))
+
+    def workspace():
+        ws = torch.empty(tk.tk_cols_workspace_bytes(n, cols), dtype=torch.uint8, device="cuda")
+        ws.view(torch.float32).fill_(float("nan"))
+        return ws
+
+    def check(grad, a, what):
+        torch.cuda.synchronize()
+        ref = tko.vjp(np.ascontiguousarray(a[:, :cols].T), np.ascontiguousarray(g[:, :cols].T), k, p, lam, mode).T
+        got = grad.cpu().numpy()
+        assert np.isfinite(got[:, :cols]).all() and rel_err(got[:, :cols], ref).max() <= TOL, (what, n)
+        assert (got[:, cols:] == -7.0).all(), (what, n)
+        grad.fill_(-7.0)
+
+    out, grad = torch.empty_like(th), torch.full_like(th, -7.0)
+    state, state2, ws, other = tk.new_state(cols), tk.new_state(cols), workspace(), workspace()
+    args = (n, cols, ld, k, p, lam, mode)
+    tk.tk_fwd_cols(th, *args, out, workspace=ws, state_out=state)
+    tk.tk_vjp_cols(th, gt, *args, grad, workspace=ws)                        # solves again
+    check(grad, x, "without state")
+    tk.tk_vjp_cols(None, gt, *args, grad, workspace=ws, state=state)
+    check(grad, x, "after a VJP without state")
+    tk.tk_fwd_cols(th2, *args, out, workspace=other, state_out=state2)
+    tk.tk_fwd_cols(th2, *args, out, workspace=ws)                            # no state asked for: the copy is left all the same
+    tk.tk_vjp_cols(None, gt, *args, grad, workspace=ws, state=state2)
+    check(grad, x2, "after a forward pass without state")
+    fresh = workspace()
+    tk.tk_vjp_cols(th, gt, *args, grad, workspace=fresh, state=state)
+    check(grad, x, "with theta and state")
+    tk.tk_vjp_cols(None, gt, *args, grad, workspace=fresh, state=state)
+    check(grad, x, "after a VJP with theta")
+    tk.tk_fwd_cols(th2, *args, out, workspace=fresh, solver=tk.TK_SOLVER_PAV)
+    tk.tk_vjp_cols(None, gt, *args, grad, workspace=fresh, state=state2)
+    check(grad, x2, "after a sorting forward pass")
