@@ -105,11 +105,20 @@ tk_status check_common(const void* theta, int64_t rows, int64_t n, int64_t k, do
 }
 
 int max_key_only_n() { return kMaxKeyOnlyN; }
+
+// What a launch ended with, as the caller sees it.  The runtime keeps the last error of a thread until it is asked for, and
+// not every launch asks (cudaLaunchKernelEx returns its own): one that is left there would be reported by the next call too.
+tk_status launched(cudaError_t e) {
+  if (e == cudaSuccess) return TK_OK;
+  (void)cudaGetLastError();
+  return TK_ERR_CUDA;
+}
 }  // namespace tk
 
 namespace {
 
 using tk::check_common;
+using tk::launched;
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -210,11 +219,11 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
     F.perm_out = nullptr;
     if (hard) { F.out = nullptr; *hard_done = true; }
     if (!hard || F.state_out) {
-      if (tk::launch_newton(F, (cudaStream_t)stream) != cudaSuccess) return TK_ERR_CUDA;
+      if ((s = launched(tk::launch_newton(F, (cudaStream_t)stream))) != TK_OK) return s;
       if (loss) loss->done = true;
     }
-    return tk::launch_perm(theta, rows, (int)n, (int)k, mode, P.perm_out, nullptr, hard ? out : nullptr, P.status,
-                           (cudaStream_t)stream) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(tk::launch_perm(theta, rows, (int)n, (int)k, mode, P.perm_out, nullptr, hard ? out : nullptr, P.status,
+                                    (cudaStream_t)stream));
   }
   // phi(x) = x with a closed-form block solve, nothing but values asked for: the threshold form needs no
   // order at all (TK_SOLVER_PAV keeps the sort)
@@ -224,7 +233,7 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
   if (by_threshold) {
     cudaError_t en = tk::launch_newton(L, (cudaStream_t)stream);
     if (loss) loss->done = true;
-    return en == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(en);
   }
   // A few very long rows (the pruning row): the same iteration with the row streamed from L2, all SMs on
   // one row at a time.  Many long rows keep the sorting pipeline, which works on all of them at once.
@@ -234,13 +243,13 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
     if (s != TK_OK) return s;
     if (opts->workspace_bytes < tk::long_newton_scratch_bytes()) return TK_ERR_WORKSPACE;
     cudaError_t eln = tk::launch_long_newton(P, opts->workspace, (cudaStream_t)stream);
-    return eln == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(eln);
   }
   if (solver == TK_SOLVER_THRESHOLD) {
     // no sort, hence no permutation to return; rows held on chip only
     if (n > tk::kMaxOnChipN || (opts && opts->perm_out)) return TK_ERR_UNSUPPORTED;
     cudaError_t et = tk::launch_thr(P, (cudaStream_t)stream);
-    return et == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(et);
   }
   if (solver == TK_SOLVER_DYKSTRA) {
     // Forward pass only: the iterate stays on chip; no row state (the iterate of a fixed number of
@@ -259,14 +268,14 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
       tk::Problem A = P;
       A.what = tk::W_ARGSORT; A.out = nullptr;
       cudaError_t ea = tk::launch_long(A, opts->workspace, nullptr, true, (cudaStream_t)stream);
-      if (ea != cudaSuccess) return TK_ERR_CUDA;
+      if (ea != cudaSuccess) return launched(ea);
       const uint32_t* keys = nullptr; const int32_t* idx = nullptr;
       tk::long_workspace_sorted(opts->workspace, rows, (int)n, &keys, &idx);
       ea = tk::launch_dykstra_cluster(P, keys, idx, (cudaStream_t)stream);
-      return ea == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+      return launched(ea);
     }
     cudaError_t ed = tk::launch_dykstra(P, (cudaStream_t)stream);
-    return ed == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(ed);
   }
   // Without a permutation to return, rows of up to 32768 elements are sorted (keys only) on chip and
   // need no workspace; one that is passed is left untouched.
@@ -275,10 +284,10 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
     s = check_workspace(opts, rows, n);
     if (s != TK_OK) return s;
     cudaError_t el = tk::launch_long(P, opts->workspace, opts->state_out, false, (cudaStream_t)stream);
-    return el == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(el);
   }
   cudaError_t e = tk::launch_on_chip(P, (cudaStream_t)stream);
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(e);
 }
 
 tk_status tk_fwd_ex(const float* theta, int64_t rows, int64_t n, int64_t k, double p,
@@ -292,7 +301,7 @@ tk_status tk_fwd_ex(const float* theta, int64_t rows, int64_t n, int64_t k, doub
   if (s != TK_OK || !st || rows == 0 || hard_done) return s;
   // the relaxed pass has left the permutation (and the row state); the hard operator replaces its output
   cudaError_t e = tk::launch_hard(theta, opts->perm_out, out, rows, (int)n, (int)k, mode, (cudaStream_t)stream);
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(e);
 }
 
 tk_status tk_fwd(const float* theta, int64_t rows, int64_t n, int64_t k, double p, double lambda,
@@ -350,7 +359,7 @@ tk_status tk_vjp(const float* theta, const float* grad_out, int64_t rows, int64_
       tk::Problem F = P;
       F.what = tk::W_FWD; F.out = nullptr; F.gout = nullptr;
       e = tk::launch_long(F, opts->workspace, nullptr, true, (cudaStream_t)stream);
-      if (e != cudaSuccess) return TK_ERR_CUDA;
+      if (e != cudaSuccess) return launched(e);
       P.state_in = tk::long_workspace_state(opts->workspace, rows, (int)n);
     }
     e = tk::launch_vjp_state_long(P, tk::long_workspace_partials(opts->workspace, rows, (int)n),
@@ -361,7 +370,7 @@ tk_status tk_vjp(const float* theta, const float* grad_out, int64_t rows, int64_
   } else {
     e = tk::launch_on_chip(P, (cudaStream_t)stream);
   }
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(e);
 }
 
 tk_status tk_jvp(const float* theta, const float* tangent, int64_t rows, int64_t n, int64_t k,
@@ -392,7 +401,7 @@ tk_status tk_jvp(const float* theta, const float* tangent, int64_t rows, int64_t
     e = tk::launch_vjp_state_long(P, tk::long_workspace_partials(opts->workspace, rows, (int)n),
                                   (cudaStream_t)stream);
   }
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(e);
 }
 
 tk_status tk_topk_loss(const float* theta, const int32_t* target, int64_t rows, int64_t n, int64_t k,
@@ -413,7 +422,7 @@ tk_status tk_topk_loss(const float* theta, const int32_t* target, int64_t rows, 
   const int vec4 = (n % 4 == 0) && aligned16(theta) && aligned16(grad);
   cudaError_t e = tk::launch_loss(theta, target, grad, loss, rows, (int)n, p, lambda, q4, qm1, vec4,
                                   (cudaStream_t)stream);
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(e);
 }
 
 // ---- the operator along the slow axis.  p = 2 and p = 4/3, columns of up to cols_direct_max_n() rows: kernels that work
@@ -463,15 +472,15 @@ tk_status tk_fwd_cols(const float* theta, int64_t n, int64_t cols, int64_t ld, i
     P.what = tk::W_FWD;
     P.state_out = opts->state_out;
     P.status = opts->status_out;
-    return tk::launch_cols_fwd(P, ld, ld, slab[0], st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(tk::launch_cols_fwd(P, ld, ld, slab[0], st));
   }
   float* theta_t = slab[direct ? 2 : 0];
-  if (tk::launch_transpose(theta, n, cols, ld, theta_t, n, direct ? slab[0] : nullptr, st) != cudaSuccess) return TK_ERR_CUDA;
+  if ((s = launched(tk::launch_transpose(theta, n, cols, ld, theta_t, n, direct ? slab[0] : nullptr, st))) != TK_OK) return s;
   tk_opts inner = *opts;
   inner.workspace = nullptr; inner.workspace_bytes = 0;
   s = tk_fwd_ex(theta_t, cols, n, k, p, lambda, mode, slab[1], &inner, stream);
   if (s != TK_OK) return s;
-  return tk::launch_transpose(slab[1], cols, n, n, out, ld, nullptr, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(tk::launch_transpose(slab[1], cols, n, n, out, ld, nullptr, st));
 }
 
 tk_status tk_vjp_cols(const float* theta, const float* grad_out, int64_t n, int64_t cols, int64_t ld,
@@ -498,22 +507,21 @@ tk_status tk_vjp_cols(const float* theta, const float* grad_out, int64_t n, int6
       tk::Problem F = P;
       F.what = tk::W_FWD;
       F.state_out = reinterpret_cast<tk_rowstate*>(slab[1]);
-      if (tk::launch_cols_fwd(F, ld, ld, slab[0], st) != cudaSuccess) return TK_ERR_CUDA;
+      if ((s = launched(tk::launch_cols_fwd(F, ld, ld, slab[0], st))) != TK_OK) return s;
       P.state_in = F.state_out;
     }
     P.gout = grad_out;
     P.out = grad_theta;
     P.what = tk::W_VJP;
-    return tk::launch_cols_vjp(P, reuse ? cols : ld, ld, ld, reuse || !opts->state_out ? nullptr : slab[0], st) == cudaSuccess
-               ? TK_OK : TK_ERR_CUDA;
+    return launched(tk::launch_cols_vjp(P, reuse ? cols : ld, ld, ld, reuse || !opts->state_out ? nullptr : slab[0], st));
   }
-  if (!reuse && tk::launch_transpose(theta, n, cols, ld, slab[0], n, nullptr, st) != cudaSuccess) return TK_ERR_CUDA;
-  if (tk::launch_transpose(grad_out, n, cols, ld, slab[1], n, nullptr, st) != cudaSuccess) return TK_ERR_CUDA;
+  if (!reuse && (s = launched(tk::launch_transpose(theta, n, cols, ld, slab[0], n, nullptr, st))) != TK_OK) return s;
+  if ((s = launched(tk::launch_transpose(grad_out, n, cols, ld, slab[1], n, nullptr, st))) != TK_OK) return s;
   tk_opts inner = *opts;
   inner.workspace = nullptr; inner.workspace_bytes = 0;
   s = tk_vjp(slab[0], slab[1], cols, n, k, p, lambda, mode, slab[2], &inner, stream);
   if (s != TK_OK) return s;
-  return tk::launch_transpose(slab[2], cols, n, n, grad_theta, ld, nullptr, st) == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(tk::launch_transpose(slab[2], cols, n, n, grad_theta, ld, nullptr, st));
 }
 
 // ---- any sorted w: relaxed linear maximisation over the permutahedron P(w)
@@ -536,7 +544,7 @@ static tk_status run_w(const float* theta, const float* w, const float* grad_out
   P.what = what;
   if (opts) P.status = opts->status_out;
   cudaError_t e = tk::launch_w(P, w, w_rows, (cudaStream_t)stream);
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(e);
 }
 
 tk_status tk_fwd_w(const float* theta, const float* w, int64_t rows, int64_t n, int64_t w_rows, double p,
@@ -567,16 +575,16 @@ tk_status tk_argsort(const float* theta, int64_t rows, int64_t n, int mode, int3
   // a longer latency on few rows; 2097 x 8000: 346 and 394)
   if (n > 64 && n <= 4096) {
     cudaError_t ep = tk::launch_perm(theta, rows, (int)n, 1, mode, perm_out, sorted_out, nullptr, P.status, (cudaStream_t)stream);
-    return ep == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(ep);
   }
   if (n > tk::kMaxOnChipN) {
     tk_status s = check_workspace(opts, rows, n);
     if (s != TK_OK) return s;
     cudaError_t el = tk::launch_long(P, opts->workspace, nullptr, true, (cudaStream_t)stream);
-    return el == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+    return launched(el);
   }
   cudaError_t e = tk::launch_on_chip(P, (cudaStream_t)stream);
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return launched(e);
 }
 
 }  // extern "C"

@@ -29,6 +29,8 @@ cudaError_t launch_long(const Problem& P, void* workspace, tk_rowstate* state_ds
 tk_status check_common(const void* theta, int64_t rows, int64_t n, int64_t k, double p, double lambda,
                        int mode, int* q4, double* qm1);
 int max_key_only_n();
+// the status of a launch, the runtime's own record of an error cleared (tk_api.cu)
+tk_status launched(cudaError_t e);
 }  // namespace tk
 
 namespace {
@@ -79,7 +81,8 @@ extern "C" tk_status tk_fwd_noalloc(const float* theta, int64_t rows, int64_t n,
   if (tk::long_workspace_bytes(rows, (int)n) > kScratchBytes) return TK_ERR_WORKSPACE;
 
   void* scratch = nullptr;
-  if (scratch_address(&scratch) != cudaSuccess) return TK_ERR_CUDA;
+  const tk_status as = tk::launched(scratch_address(&scratch));
+  if (as != TK_OK) return as;
 
   tk::Problem P{};
   P.theta = theta;
@@ -92,6 +95,5 @@ extern "C" tk_status tk_fwd_noalloc(const float* theta, int64_t rows, int64_t n,
   // Nothing in the scratch has to start at zero: every word a kernel of this pipeline reads
   // (sort buffers, histograms, prefix sums, tile totals, row state) is written earlier in the
   // same call, so the previous call's contents are simply overwritten.
-  cudaError_t e = tk::launch_long(P, scratch, nullptr, false, (cudaStream_t)stream);
-  return e == cudaSuccess ? TK_OK : TK_ERR_CUDA;
+  return tk::launched(tk::launch_long(P, scratch, nullptr, false, (cudaStream_t)stream));
 }

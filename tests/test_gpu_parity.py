@@ -1296,3 +1296,31 @@ def test_slow_axis_vjp_without_theta_reads_the_last_theta_given(n, p, mode):
     tk.tk_fwd_cols(th2, *args, out, workspace=fresh, solver=tk.TK_SOLVER_PAV)
     tk.tk_vjp_cols(None, gt, *args, grad, workspace=fresh, state=state2)
     check(grad, x2, "after a sorting forward pass")
+
+
+def test_a_failed_launch_is_reported_once():
+    """A launch that CUDA refuses (here: into a stream whose capture has been invalidated on the host) is TK_ERR_CUDA for that
+    call; the next call, which launches, must not report it again."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.12")
+    rows, n, k = 5, 1500, 40
+    th = torch.from_numpy(rows_of(n, rows, 41, 1.0)).cuda()
+    out, ref = torch.empty_like(th), torch.empty_like(th)
+    tk.tk_fwd_ex(th, rows, n, k, 2.0, 1.0, tk.TK_MASK, ref, solver=tk.TK_SOLVER_PAV)
+    torch.cuda.synchronize()
+    perm = torch.empty(rows, n, dtype=torch.int32, device="cuda")
+    calls = [lambda: tk.tk_fwd(th, rows, n, k, 2.0, 1.0, tk.TK_MASK, out),
+             lambda: tk.tk_argsort(th, rows, n, tk.TK_MASK, perm)]
+    stream = torch.cuda.Stream()
+    handle, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    for call in calls:
+        assert rt.cudaStreamBeginCapture(handle, 2) == 0
+        assert rt.cudaStreamSynchronize(handle) != 0            # not allowed during a capture: it is invalid from here on
+        with torch.cuda.stream(stream), pytest.raises(tk.TkError) as e:
+            call()
+        assert e.value.status == tk.TK_ERR_CUDA
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) != 0 and not graph.value
+        rt.cudaGetLastError()
+        tk.tk_fwd_ex(th, rows, n, k, 2.0, 1.0, tk.TK_MASK, out, solver=tk.TK_SOLVER_PAV)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
