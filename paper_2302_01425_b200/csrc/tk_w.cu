@@ -85,6 +85,8 @@ struct WRow {
   const double* p2;               // p = 4/3: of d^2, d^3, w
   const double* p3;
   const double* pw;
+  const float* s;                 // p = 4/3: the sorted keys, and whether they lie far apart
+  bool wide;
 };
 
 template <int E>
@@ -102,8 +104,15 @@ __device__ __forceinline__ double w_block_value(const WRow& A, int a, int b, dou
   if (!Q4) return S1 / N;
   const double W = w_range<E>(A.pw, a, b), S2 = w_range<E>(A.p2, a, b), S3 = w_range<E>(A.p3, a, b);
   const double mu = S1 / N;
-  const double M2 = fmax(S2 - S1 * mu, 0.0);
-  const double M3 = S3 - 3.0 * mu * S2 + 2.0 * mu * mu * S1;
+  double M2 = fmax(S2 - S1 * mu, 0.0), M3 = S3 - 3.0 * mu * S2 + 2.0 * mu * mu * S1;
+  if (A.wide) {
+    // The moments about the block's mean are differences of prefix sums about the row's pivot: noise, for keys close together
+    // and far from it (entries masked with -1e9).  The block's own keys bound them: within a range of r, N r^2 / 4 and
+    // N r^3 / (6 sqrt 3).  Without that the noise decides which blocks pool, and the joins take many more rounds.
+    const double r = (double)A.s[wp<E>(a)] - (double)A.s[wp<E>(b - 1)], nr2 = N * r * r, top3 = 0.0963 * nr2 * r;
+    M2 = fmin(M2, 0.25 * nr2);
+    M3 = fmin(fmax(M3, -top3), top3);
+  }
   // sum (g - d_i)^3 + lam^3 W = 0 with g = mu + h:  N h^3 + 3 M2 h - M3 + lam^3 W = 0
   return mu + w_cubic_root(N, M2, lam3 * W - M3);
 }
@@ -171,7 +180,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
   const int base = lig * E;                                       // its first rank
   const int sbase = rbase + lig * (E + 1);                        // and that rank's slot
   WRow A;
-  A.val = val + rbase; A.p1 = p1 + rbase; A.p2 = p2 + rbase; A.p3 = p3 + rbase; A.pw = pw + rbase;
+  A.val = val + rbase; A.p1 = p1 + rbase; A.p2 = p2 + rbase; A.p3 = p3 + rbase; A.pw = pw + rbase; A.s = s + rbase; A.wide = false;
   // row of element e of the team's rows: exact for e < 2^16 (n == 1 would overflow the multiplier)
   const uint32_t magic = n > 1 ? 0xffffffffu / (uint32_t)n + 1u : 0u;
   auto row_of = [&](int e) -> int { return R == 1 ? 0 : (n > 1 ? (int)__umulhi((uint32_t)e, magic) : e); };
@@ -179,7 +188,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
   overlap_wait();
   // ---- theta as it lies in memory, w by rank (in the keys' array, which is free until the sort is done).  Every
   // load is unconditional (past the end the last element again), so the loads of a lane are all in flight at once
-  bool bad = false;
+  int flags = 0;
   if (VJP && 32 * tid < total)                                    // the cotangent is wanted after the solve: into L2 by then
     asm volatile("prefetch.global.L2 [%0];" ::"l"(P.gout + first + 32 * tid));
   {
@@ -189,7 +198,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
     for (int it = 0; it < E; ++it) v[it] = src[min(tid + it * TL, total - 1)];
 #pragma unroll
     for (int it = 0; it < E; ++it) {
-      bad |= !(fabsf(v[it]) < INFINITY);
+      if (!(fabsf(v[it]) < INFINITY)) flags = TK_FLAG_NONFINITE;
       if (tid + it * TL < total) xs[tid + it * TL] = v[it];
     }
     if (w_shared) {
@@ -251,11 +260,20 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
   }
   w_sync<W>();                                                    // the rows have been taken out of p1
 
-  // ---- 2. prefix sums about a pivot (a key near the middle), singleton values
-  const int plane = (n / 2) / E;                                  // the lane whose first key it is
-  float pivf = __shfl_sync(0xffffffffu, r[0], W == 1 ? rl * G + plane : plane & 31);
+  // ---- 2. prefix sums about a pivot (a key near the middle), singleton values.  p = 4/3: the key of rank n / 2 itself.  The
+  // first key of that rank's lane is up to 15 ranks away, in a row of a few keys the largest one; the third powers of keys
+  // far below it cancel to noise, and one far key decides about all the others: (x, -1e9, -1e9) came out thousands off.
+  // (p = 2 has no powers to lose: 3 % slower with it, 8192 x 512.)
+  const int plane = (n / 2) / E;
+  float pivf = r[0];
+  if (Q4) {
+#pragma unroll
+    for (int i = 1; i < E; ++i)
+      if (i == (n / 2) % E) pivf = r[i];
+  }
+  if (W > 1 && tid == plane) redd[0] = (double)pivf;
+  pivf = __shfl_sync(0xffffffffu, pivf, W == 1 ? rl * G + plane : plane & 31);
   if (W > 1) {
-    if (tid == plane) redd[0] = (double)r[0];
     __syncthreads();
     pivf = (float)redd[0];
     __syncthreads();
@@ -271,6 +289,10 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
       if ((lig & (G - 1)) >= o) inc += up;
     }
     double before = inc - mine;
+    if (Q4) {                                                     // (that loses the sum of third powers before a lane of far keys)
+      before = __shfl_up_sync(0xffffffffu, inc, 1, G);
+      if ((lig & (G - 1)) == 0) before = 0.0;
+    }
     if (W > 1) {
       if (lane == 31) redd[warp] = inc;
       __syncthreads();
@@ -283,7 +305,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
   const float* wl = s + (w_shared ? 0 : rbase) + lig * (E + 1);
   {
     constexpr int NS = Q4 ? 4 : 1;
-    double run[NS];
+    double run[NS], reach = 0.0;                                  // p = 4/3: this lane's largest distance from the pivot
 #pragma unroll
     for (int q = 0; q < NS; ++q) run[q] = 0.0;
 #pragma unroll
@@ -294,6 +316,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
         val[sbase + i] = h;
         if (!Q4) { run[0] += h; p1[sbase + i] = run[0]; }
         else {
+          if (i == 0 || i == cl - 1) reach = fmax(reach, fabs(d));
           run[0] += d; run[NS > 1 ? 1 : 0] += d * d; run[NS > 2 ? 2 : 0] += d * d * d; run[NS > 3 ? 3 : 0] += wi;
           p1[sbase + i] = run[0]; p2[sbase + i] = run[NS > 1 ? 1 : 0];
           p3[sbase + i] = run[NS > 2 ? 2 : 0]; pw[sbase + i] = run[NS > 3 ? 3 : 0];
@@ -301,7 +324,13 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
       }
     }
     lanes_before(run[0], p1);
-    if (Q4) { lanes_before(run[NS > 1 ? 1 : 0], p2); lanes_before(run[NS > 2 ? 2 : 0], p3); lanes_before(run[NS > 3 ? 3 : 0], pw); }
+    if (Q4) {
+      lanes_before(run[NS > 1 ? 1 : 0], p2); lanes_before(run[NS > 2 ? 2 : 0], p3); lanes_before(run[NS > 3 ? 3 : 0], pw);
+      // (within 256 lambda of the pivot the moments' noise is below 1e-8 N lambda^3, and a row does without their bounds)
+      const bool wide = !(reach <= 256.0 * lam);
+      if (W > 1) A.wide = __syncthreads_or(wide) != 0;
+      else A.wide = (__ballot_sync(0xffffffffu, wide) >> (rl * G) & (0xffffffffu >> (32 - G))) != 0u;
+    }
   }
   w_sync<W>();                                                    // w has been read everywhere
 #pragma unroll
@@ -672,7 +701,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
       }
     }
   }
-  if (bad && P.status) atomicOr(P.status, TK_FLAG_NONFINITE);
+  if (flags && P.status) atomicOr(P.status, flags);
 }
 
 template <int E, int G, int W, bool Q4, bool VJP>

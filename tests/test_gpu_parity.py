@@ -1324,3 +1324,34 @@ def test_a_failed_launch_is_reported_once():
         tk.tk_fwd_ex(th, rows, n, k, 2.0, 1.0, tk.TK_MASK, out, solver=tk.TK_SOLVER_PAV)
         torch.cuda.synchronize()
         assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("p", [2.0, P43])
+@pytest.mark.parametrize("n", [2, 3, 5, 8, 9, 16, 17, 33, 100, 256, 257, 1000, 2048])
+def test_general_sorted_w_with_masked_entries(n, p):
+    """Entries masked with -1e9, all but one of a row (the pivot of the sums is one of the masked keys), and a part of it.
+    The sums carry differences of 1e9 then: an error of 1e9 u, u the unit roundoff of fp64, in the distance of a key from its
+    block, and three times that relative to lambda at p = 4/3 -- times n for the prefix sums' roundings.  Which keys pool
+    does not depend on it where equal keys pool among themselves: the cotangent in w must be right."""
+    from oracle import tko
+    rows, lam = 19, 1.0
+    x = rows_of(n, rows, 17000 + n, 1.0)
+    few = np.full_like(x, -1e9)
+    few[:, n // 3] = x[:, 0]
+    part = x.copy()
+    part[:, n // 4: n // 2 + 1] = -1e9
+    w = (np.arange(n, 0, -1) / n).astype(np.float32)
+    g = wl.cotangent_like(x, 17100 + n)
+    for name, a in (("few", few), ("part", part)):
+        th, wt, gt = (torch.from_numpy(v).cuda() for v in (a, w, g))
+        out, grad, gw = (torch.full((rows, n), float("nan"), device="cuda") for _ in range(3))
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        tk.tk_fwd_w(th, wt, rows, n, p, lam, out, status_out=status)
+        tk.tk_vjp_w(th, wt, gt, rows, n, p, lam, grad, grad_w=gw, status_out=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        gref, gwref = tko.vjp_w(a, w, g, p, lam, with_w=True)
+        tol = 1e-5 + 3 * n * 1e9 * 2.0 ** -53 / lam * (1.0 if name == "few" else n)
+        for what, got, ref in (("forward", out, tko.fwd_w(a, w, p, lam)), ("vjp", grad, gref), ("vjp in w", gw, gwref)):
+            e = np.abs(got.cpu().numpy() - ref) / np.maximum(1.0, np.abs(ref))
+            assert e.max() <= tol, f"{name} n={n} {what}: {e.max()} above {tol}"
