@@ -505,6 +505,7 @@ __global__ void __launch_bounds__(WGeom<E, W, Q4>::THREADS, WGeom<E, W, Q4>::MIN
       }
       if (!(wide ? __syncthreads_or(act) : __any_sync(0xffffffffu, act))) break;
     }
+    if (act) flags |= TK_FLAG_NOT_CONVERGED;                      // (the cap)
     if (wide) __syncthreads(); else __syncwarp();
   }
 
