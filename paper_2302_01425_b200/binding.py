@@ -7,20 +7,38 @@ fails loudly when the library has not been built.
 
 A call goes through _tk_bind (csrc/host/tk_bind.cpp: the same checks and the same call in C++, 1 us
 instead of 8); what it does not take -- no library bound yet, or an argument that fails a check --
-it hands back, and the ctypes code below loads the library or raises the error.
+it hands back, and the ctypes code below loads the library or raises the error.  Without a _tk_bind
+built for this Python and this torch every call takes the ctypes code, and load() says so.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
+import warnings
 from typing import Optional
 
 import torch
 
-try:
-    from . import _tk_bind as _native
-except ImportError:             # not built yet: every call takes the ctypes code
-    _native = None
+from .build import bind_path
+
+
+def _load_native(path: str):
+    """_tk_bind from that file, or None and the reason."""
+    if not os.path.exists(path):
+        return None, "not built"
+    loader = importlib.machinery.ExtensionFileLoader("_tk_bind", path)
+    spec = importlib.util.spec_from_file_location("_tk_bind", path, loader=loader)
+    try:
+        module = importlib.util.module_from_spec(spec)
+        loader.exec_module(module)
+    except ImportError as e:
+        return None, str(e)
+    return module, None
+
+
+_native, _native_missing = _load_native(bind_path())
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libtk.so")
@@ -115,7 +133,10 @@ def load() -> ctypes.CDLL:
     lib.tk_argsort.restype = ci
     lib.tk_argsort.argtypes = [vp, i64, i64, ci, vp, vp, ctypes.POINTER(TkOpts), vp]
     _lib = lib
-    if _native is not None:
+    if _native is None:
+        warnings.warn(f"{bind_path()}: {_native_missing}; calls go through ctypes, 8 us of host time each "
+                      "(python -m paper_2302_01425_b200.build)", RuntimeWarning, stacklevel=2)
+    else:
         _native.bind(*(ctypes.cast(getattr(lib, f), vp).value for f in _NATIVE_ENTRIES))
     return lib
 

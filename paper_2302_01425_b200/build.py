@@ -12,13 +12,13 @@ import glob
 import os
 import subprocess
 import sys
+import warnings
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 LIB = os.path.join(_PKG, "libtk.so")
 LIB_BOUNDS = os.path.join(_PKG, "libtk_bounds.so")
-BIND = os.path.join(_PKG, "_tk_bind.so")
 BIND_SRC = os.path.join(CSRC, "host", "tk_bind.cpp")
 
 NVCC_FLAGS = [
@@ -40,17 +40,25 @@ def _stale(lib: str = LIB) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def bind_path() -> str:
+    """Where the C++ half of the binding lies.  It reads tensors by the layout of one torch and objects by that of one Python,
+    and neither is stable: both versions are in its name, and another's is not picked up."""
+    import torch
+    return os.path.join(_PKG, f"_tk_bind.{sys.implementation.cache_tag}-torch{torch.__version__}.so")
+
+
 def build_bind(force: bool = False) -> str:
     """The C++ half of the binding (argument marshalling), against torch's headers and libraries."""
+    out = bind_path()
     header = os.path.join(_ROOT, "include", "tk.h")
-    if not force and os.path.exists(BIND) and all(os.path.getmtime(f) <= os.path.getmtime(BIND) for f in (BIND_SRC, header)):
-        return BIND
+    if not force and os.path.exists(out) and all(os.path.getmtime(f) <= os.path.getmtime(out) for f in (BIND_SRC, header)):
+        return out
     import sysconfig
     import torch
     from torch.utils import cpp_extension
     base = os.path.join(os.path.dirname(torch.__file__))
     cuda = cpp_extension.CUDA_HOME or "/usr/local/cuda"
-    tmp = BIND + f".tmp{os.getpid()}"
+    tmp = out + f".tmp{os.getpid()}"
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-w",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"]
     for d in [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
@@ -58,16 +66,24 @@ def build_bind(force: bool = False) -> str:
         cmd += ["-I", d]
     cmd += ["-o", tmp, BIND_SRC, "-L", os.path.join(base, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     subprocess.run(cmd, check=True)
-    os.replace(tmp, BIND)
-    return BIND
+    os.replace(tmp, out)
+    return out
 
 
 def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> str:
-    if not bounds:
-        build_bind(force)
     lib = LIB_BOUNDS if bounds else LIB
-    if not force and not _stale(lib):
-        return lib
+    if force or _stale(lib):
+        _build_library(lib, verbose, bounds)
+    if not bounds:
+        try:
+            build_bind(force)
+        except (ImportError, OSError, subprocess.CalledProcessError) as e:      # the library serves without it
+            warnings.warn(f"the C++ half of the binding could not be built ({e}): calls will go through ctypes, "
+                          "8 us of host time each", RuntimeWarning, stacklevel=2)
+    return lib
+
+
+def _build_library(lib: str, verbose: bool, bounds: bool) -> None:
     nvcc = os.environ.get("NVCC", "nvcc")
     tmp = lib + f".tmp{os.getpid()}"
     cmd = [nvcc] + NVCC_FLAGS
@@ -78,7 +94,6 @@ def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> s
     cmd += ["-I", os.path.join(_ROOT, "include"), "-I", CSRC, "-o", tmp] + sources()
     subprocess.run(cmd, check=True)
     os.replace(tmp, lib)
-    return lib
 
 
 if __name__ == "__main__":
