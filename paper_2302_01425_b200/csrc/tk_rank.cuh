@@ -112,7 +112,7 @@ __device__ __forceinline__ int rank_find(const float* s, int n, float key) {
 // Ranks of equal keys in index order.  rk[i]: what rank_find returned for element lig + T i of this lane's row (its
 // place in the run's order is added); s: the row's sorted keys.  work: max(R * NP, kRkList + 1) words of shared memory.
 // All lanes of the team call it.  Up to kRkList elements with equals: listed, and each counts the earlier ones of its
-// run.  More: the row is walked 32 elements at a time in index order (128 steps of about 600 cycles at n = 4096).
+// run.  More: the row is walked in index order.
 constexpr int kRkList = 64;
 
 template <int G, int W>
@@ -148,30 +148,67 @@ __device__ __forceinline__ void rank_ties(int (&rk)[kRkE], const float* s, int n
     rk_sync<W>();
     return;
   }
+  // Elements in index order, 32 at a time: a step finds which of them are equal, reads how many of their run have been
+  // placed, and adds its own.
   rk_sync<W>();
-  int* cnt = work;                              // how many of a run have been placed
-  for (int i = tid; i < Geom::R * Geom::NP; i += Geom::TL) cnt[i] = 0;
-  rk_sync<W>();
+  uint16_t* cnt = reinterpret_cast<uint16_t*>(work);              // [R * N], by rank: how many of a run have been placed
+  for (int i = tid; i < Geom::R * Geom::N / 2; i += Geom::TL) work[i] = 0;
+  if constexpr (W == 1) {
+    __syncwarp();
 #pragma unroll
-  for (int i = 0; i < kRkE; ++i) {
+    for (int i = 0; i < kRkE; ++i) {
+      const bool in = lig + Geom::T * i < n;
+      const int slot = rl * Geom::N + rk[i];
+      const unsigned same = __match_any_sync(0xffffffffu, in ? slot : -1 - lane);
+      const int before = __popc(same & ((1u << lane) - 1u));
+      int placed = 0;
+      if (in) placed = cnt[slot];
+      __syncwarp();
+      if (in) {
+        if (before == 0) cnt[slot] = (uint16_t)(placed + __popc(same));
+        rk[i] = min(rk[i] + placed + before, n - 1);
+      }
+      __syncwarp();
+    }
+  } else {
+    // Each warp takes 512 consecutive elements (through shared memory) and finds the equal ones of all its steps first; then
+    // the warps take turns, and a turn is 16 times read, add, write.  (Us, a third of the entries masked, every step of all
+    // warps in turn with a block barrier after it / here: argsort 524 x 4000 85 / 52, with a 64-bit network 47; permutation
+    // and values 256 x 8192 204 / 121.  One warp per row has no barriers to save, and the extra passes cost it 17 %.)
+    uint16_t* ranks = cnt + Geom::N;                              // [N], by element
+#pragma unroll
+    for (int i = 0; i < kRkE; ++i) ranks[lig + Geom::T * i] = (uint16_t)rk[i];
+    __syncthreads();
+    uint16_t* mine = ranks + warp * (32 * kRkE) + lane;
+    const int left = n - warp * (32 * kRkE) - lane;               // this lane's elements of the warp's: 32 i < left
+    int at[kRkE];                               // rank of the run | earlier ones among the 32 | the run's share of them
+#pragma unroll
+    for (int i = 0; i < kRkE; ++i) {
+      const int r = mine[32 * i];
+      const unsigned same = __match_any_sync(0xffffffffu, 32 * i < left ? r : -1 - lane);
+      at[i] = r | __popc(same & ((1u << lane) - 1u)) << 16 | __popc(same) << 24;
+    }
 #pragma unroll 1
     for (int w = 0; w < W; ++w) {
       if (w == warp) {
-        const bool in = lig + Geom::T * i < n;
-        const int slot = rl * Geom::NP + rk_slot<G, W>(rk[i]);
-        const unsigned same = __match_any_sync(0xffffffffu, in ? slot : -1 - lane);
-        const int before = __popc(same & ((1u << lane) - 1u));
-        int placed = 0;
-        if (in) placed = cnt[slot];
-        __syncwarp();
-        if (in) {
-          if (before == 0) cnt[slot] = placed + __popc(same);
-          rk[i] = min(rk[i] + placed + before, n - 1);
+#pragma unroll
+        for (int i = 0; i < kRkE; ++i) {
+          const int r = at[i] & 0xffff, before = at[i] >> 16 & 0xff;
+          int placed = 0;
+          if (32 * i < left) placed = cnt[r];
+          __syncwarp();
+          if (32 * i < left && before == 0) cnt[r] = (uint16_t)(placed + (at[i] >> 24));
+          at[i] = min(r + placed + before, n - 1);
+          __syncwarp();
         }
-        __syncwarp();
       }
-      if (W > 1) __syncthreads();
+      __syncthreads();
     }
+#pragma unroll
+    for (int i = 0; i < kRkE; ++i) mine[32 * i] = (uint16_t)at[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kRkE; ++i) rk[i] = ranks[lig + Geom::T * i];
   }
   rk_sync<W>();
 }
