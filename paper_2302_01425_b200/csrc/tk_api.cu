@@ -211,19 +211,16 @@ static tk_status fwd_relaxed(const float* theta, int64_t rows, int64_t n, int64_
   tk::Problem L = P;                            // what the threshold form is asked for
   if (loss) { L.loss = loss->loss; L.target = loss->target; }
   // A permutation from AUTO: the order comes from the keys-only sort, the relaxed values and the row state from the
-  // threshold form, which needs no order.  One kernel that sorts 64-bit words and solves on them (and another that makes
-  // the hard output) stays faster up to 32 elements only: 699050 x 24, p = 2: 269 us and 270; 262144 x 64: 221 and 118;
-  // 4194 x 4000: 420 and 265.  A hard output needs the row state alone.
+  // threshold form, started at the k-th key of that order.  One kernel that sorts 64-bit words and solves on them (and
+  // another that makes the hard output) stays faster up to 32 elements only: 699050 x 24, p = 2: 269 us and 270; 262144 x 64:
+  // 221 and 118; 4194 x 4000: 420 and 265.  A hard output needs the row state alone.
   if (solver == TK_SOLVER_AUTO && P.perm_out && qm1 == 0.0 && n > 32 && n <= tk::perm_max_n()) {
-    tk::Problem F = L;
-    F.perm_out = nullptr;
-    if (hard) { F.out = nullptr; *hard_done = true; }
-    if (!hard || F.state_out) {
-      if ((s = launched(tk::launch_newton(F, (cudaStream_t)stream))) != TK_OK) return s;
-      if (loss) loss->done = true;
-    }
-    return launched(tk::launch_perm(theta, rows, (int)n, (int)k, mode, P.perm_out, nullptr, hard ? out : nullptr, P.status,
-                                    (cudaStream_t)stream));
+    s = launched(tk::launch_perm(theta, rows, (int)n, (int)k, mode, P.perm_out, nullptr, hard ? out : nullptr, P.status,
+                                 (cudaStream_t)stream));
+    if (s != TK_OK) return s;
+    if (hard) { L.out = nullptr; *hard_done = true; }
+    if (loss) loss->done = true;
+    return hard && !L.state_out ? TK_OK : launched(tk::launch_newton(L, (cudaStream_t)stream));
   }
   // phi(x) = x with a closed-form block solve, nothing but values asked for: the threshold form needs no
   // order at all (TK_SOLVER_PAV keeps the sort)

@@ -1355,3 +1355,53 @@ def test_general_sorted_w_with_masked_entries(n, p):
         for what, got, ref in (("forward", out, tko.fwd_w(a, w, p, lam)), ("vjp", grad, gref), ("vjp in w", gw, gwref)):
             e = np.abs(got.cpu().numpy() - ref) / np.maximum(1.0, np.abs(ref))
             assert e.max() <= tol, f"{name} n={n} {what}: {e.max()} above {tol}"
+
+
+@pytest.mark.parametrize("p", [2.0, P43])
+@pytest.mark.parametrize("n", [33, 64, 65, 400, 1025, 4097, 8192])
+def test_permutation_with_rows_that_start_far_from_the_root(n, p):
+    """Values and row state beside a permutation start at the k-th key of that order: rows whose moments say nothing about it
+    (masked entries, ratios of normals, lambda far below the spacing of the keys), ties at that key, every mode."""
+    from oracle import tko
+    from parity import rel_err, TOL
+    rows = 40 if n <= 65 else 6
+    base = rows_of(n, rows, 18000 + n, 1.0)
+    masked = base.copy()
+    masked[:, ::3] = -1e9
+    tails = (base / np.maximum(np.abs(rows_of(n, rows, 18100 + n, 1.0)), 1e-3)).astype(np.float32)
+    tied = (np.round(base * 4) / 4).astype(np.float32)
+    for name, x, lam in (("masked", masked, 1.0), ("tails", tails, 0.05), ("small lambda", base, 1e-4), ("tied", tied, 0.3)):
+        th = torch.from_numpy(x).cuda()
+        for mode in (tk.TK_MASK, tk.TK_TOPK, tk.TK_TOPKMAG):
+            if mode != tk.TK_MASK and name == "masked":
+                continue                                        # (-1e9 is a value of those)
+            # (masked: no masked key selected, the oracle's third powers of 1e9 have no digits left for the others)
+            for k in sorted({1, 3, n // 5, n // 2} | (set() if name == "masked" else {n - 1, n})):
+                out, state = torch.full_like(th, float("nan")), tk.new_state(rows)
+                perm, status = torch.empty(rows, n, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+                tk.tk_fwd_ex(th, rows, n, k, p, lam, mode, out, perm_out=perm, state_out=state, status_out=status)
+                torch.cuda.synchronize()
+                assert int(status.item()) == 0, (name, mode, k)
+                assert np.array_equal(perm.cpu().numpy(), tko.argsort(x, mode)[0]), (name, mode, k)
+                assert rel_err(out.cpu().numpy(), tko.fwd(x, k, p, lam, mode)).max() <= TOL, (name, mode, k)
+                hard, state2 = torch.full_like(th, float("nan")), tk.new_state(rows)
+                tk.tk_fwd_ex(th, rows, n, k, p, lam, mode, hard, perm_out=perm, state_out=state2, flags=tk.TK_OPT_STRAIGHT_THROUGH)
+                torch.cuda.synchronize()
+                assert torch.equal(state, state2), (name, mode, k)
+                assert np.array_equal(hard.cpu().numpy(), tko.hard(x, k, mode).astype(np.float32)), (name, mode, k)
+
+
+def test_permutation_of_a_full_batch_of_short_rows():
+    """Enough rows of 61 for two lanes per row through the staging tile."""
+    from oracle import tko
+    from parity import rel_err, TOL
+    rows, n, k, lam = 60000, 61, 9, 0.05
+    x = rows_of(n, rows, 18500, 1.0)
+    x[:, ::4] = -1e9
+    th = torch.from_numpy(x).cuda()
+    out, perm = torch.full_like(th, float("nan")), torch.empty(rows, n, dtype=torch.int32, device="cuda")
+    tk.tk_fwd_ex(th, rows, n, k, P43, lam, tk.TK_MASK, out, perm_out=perm)
+    torch.cuda.synchronize()
+    pick = np.arange(0, rows, 97)
+    assert np.array_equal(perm.cpu().numpy()[pick], tko.argsort(x[pick], tk.TK_MASK)[0])
+    assert rel_err(out.cpu().numpy()[pick], tko.fwd(x[pick], k, P43, lam, tk.TK_MASK)).max() <= TOL
