@@ -530,14 +530,14 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
   nt_row_init(S, k);
   float lo = -FLT_MAX, hi = FLT_MAX;
   if (KSEL == 0) {
-    // where the order is known (P.perm_out) the k-th largest key says where to start: the root lies within one width below
+    // Where the order is known (P.perm_out) the k-th largest key says where to start: the root lies within one width below
     // it, whatever the moments say (us, permutation and values, moments / this: 524 x 4000, lambda = 0.01, p = 4/3 55 / 46,
-    // ratios of normals 196 / 48; 20971 x 100 49 / 35, a third masked 104 / 51)
-    float s_k = 0.0f;
-    if (P.perm_out && TK_IN_BOUNDS(io.first + k - 1, 1, io.extent, P.status)) {
-      s_k = io.src[min((unsigned)P.perm_out[io.first + k - 1], (unsigned)n - 1u)];
-      if (MAG) s_k = fabsf(s_k);
-    }
+    // ratios of normals 196 / 48; 20971 x 100 49 / 35, a third masked 104 / 51).
+    const bool ordered = WHAT != NT_LOSS && P.perm_out != nullptr;
+    auto kth_key = [&]() -> float {
+      if (!TK_IN_BOUNDS(io.first + k - 1, 1, io.extent, P.status)) return 0.0f;
+      return io.src[min((unsigned)P.perm_out[io.first + k - 1], (unsigned)n - 1u)];
+    };
     // sums about the row's first key: mean and spread of the keys
     const float x0 = MAG ? 0.0f : *io.src;
     float v[2] = {0.f, 0.f};
@@ -572,7 +572,8 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
       if (k == n) {                            // everything is selected
         S.piv = -FLT_MAX; S.off = -wid; S.done = true; S.noblock = true;
       } else {
-        float tau0 = (P.perm_out ? s_k : (x0 + mean_d) + zq * sd) - (Q4 ? 0.75f : 0.5f) * lam;
+        float tau0 = (x0 + mean_d) + zq * sd - (Q4 ? 0.75f : 0.5f) * lam;
+        if (ordered) tau0 = kth_key() - (Q4 ? 0.75f : 0.5f) * lam;
         if (!(fabsf(tau0) < FLT_MAX)) tau0 = x0;
         S.piv = tau0;
       }
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
       } else {
         // zq: the upper k/(2n) quantile of N(0,1); the keys of a zero-mean row are its absolute values.
         // About k keys lie above gamma + width/2 (q = 2) or gamma + 3 width/4 (q = 4).
-        const float t0 = P.perm_out ? s_k : zq * sqrtf(v[1] * inv_n);
+        const float t0 = ordered ? fabsf(kth_key()) : zq * sqrtf(v[1] * inv_n);
         float tau0 = Q4 ? t0 - 0.75f * lam * cbrtf(t0) : t0 / (1.0f + 0.5f * lam);
         if (!(tau0 > 0.0f && tau0 < FLT_MAX)) tau0 = 0.5f * t0;
         if (!(tau0 > 0.0f && tau0 < FLT_MAX)) tau0 = 1.0f;
