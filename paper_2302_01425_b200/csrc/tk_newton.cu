@@ -18,7 +18,7 @@
 //     sums t, t^2, t^3 over the inside keys; the piece's equation gives the next tau;
 //   - a step that leaves the bracket is replaced by a step of doubling length towards the root,
 //     then by bisection (of the ordered integer keys when the bracket spans many binades), and
-//     after six Newton steps in a row one such step is forced: the loop ends;
+//     after six Newton steps in a row such steps are forced, larger each time: the loop ends;
 //   - the root is accepted when a point reproduces the set of the pass before it and already
 //     solves it to rounding, or when cm |du| is rounding-sized (F has slope >= 1/lambda until
 //     it reaches an integer, so the root is then within that distance).
@@ -532,11 +532,18 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
   if (KSEL == 0) {
     // Where the order is known (P.perm_out) the k-th largest key says where to start: the root lies within one width below
     // it, whatever the moments say (us, permutation and values, moments / this: 524 x 4000, lambda = 0.01, p = 4/3 55 / 46,
-    // ratios of normals 196 / 48; 20971 x 100 49 / 35, a third masked 104 / 51).
+    // ratios of normals 196 / 48; 20971 x 100 49 / 35, a third masked 104 / 51).  Where the next key lies lower than that
+    // nothing is pooled: the start is halfway between, where the first pass sees it.  (At the k-th key's own edge rounding
+    // would decide whether it reads as pooled alone.)
     const bool ordered = WHAT != NT_LOSS && P.perm_out != nullptr;
-    auto kth_key = [&]() -> float {
-      if (!TK_IN_BOUNDS(io.first + k - 1, 1, io.extent, P.status)) return 0.0f;
-      return io.src[min((unsigned)P.perm_out[io.first + k - 1], (unsigned)n - 1u)];
+    auto key_of_rank = [&](int rank) -> float {
+      if (!TK_IN_BOUNDS(io.first + rank, 1, io.extent, P.status)) return 0.0f;
+      const float x = io.src[min((unsigned)P.perm_out[io.first + rank], (unsigned)n - 1u)];
+      return MAG ? fabsf(x) : x;
+    };
+    auto start_of = [&](float inside, float low) -> float {       // low: at most the k-th key's own value, unpooled
+      const float next = key_of_rank(k);
+      return low > next ? 0.5f * (low + next) : inside;
     };
     // sums about the row's first key: mean and spread of the keys
     const float x0 = MAG ? 0.0f : *io.src;
@@ -573,7 +580,10 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
         S.piv = -FLT_MAX; S.off = -wid; S.done = true; S.noblock = true;
       } else {
         float tau0 = (x0 + mean_d) + zq * sd - (Q4 ? 0.75f : 0.5f) * lam;
-        if (ordered) tau0 = kth_key() - (Q4 ? 0.75f : 0.5f) * lam;
+        if (ordered) {
+          const float s_k = key_of_rank(k - 1);
+          tau0 = start_of(s_k - (Q4 ? 0.75f : 0.5f) * lam, s_k - lam);
+        }
         if (!(fabsf(tau0) < FLT_MAX)) tau0 = x0;
         S.piv = tau0;
       }
@@ -584,8 +594,9 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
       } else {
         // zq: the upper k/(2n) quantile of N(0,1); the keys of a zero-mean row are its absolute values.
         // About k keys lie above gamma + width/2 (q = 2) or gamma + 3 width/4 (q = 4).
-        const float t0 = ordered ? fabsf(kth_key()) : zq * sqrtf(v[1] * inv_n);
+        const float t0 = ordered ? key_of_rank(k - 1) : zq * sqrtf(v[1] * inv_n);
         float tau0 = Q4 ? t0 - 0.75f * lam * cbrtf(t0) : t0 / (1.0f + 0.5f * lam);
+        if (ordered) tau0 = start_of(tau0, Q4 ? t0 - lam * cbrtf(t0) : t0 / (1.0f + lam));
         if (!(tau0 > 0.0f && tau0 < FLT_MAX)) tau0 = 0.5f * t0;
         if (!(tau0 > 0.0f && tau0 < FLT_MAX)) tau0 = 1.0f;
         S.piv = tau0;
