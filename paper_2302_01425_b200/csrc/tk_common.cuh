@@ -86,9 +86,13 @@ inline int sm_count() {
 // data that nobody writes while the grid exists).  The kernel after them may start once all their blocks have called
 // overlap_next() (or ended).  Where that is matters: blocks of the next grid that settle while most of this one's are still
 // at work crowd the SMs that have room, and their share of the work stays there.
-// After the row has been read and the starting guess is known was the best place for the Newton kernel and its VJP
-// (forward + VJP, us: at the kernel's start / there: 10007 x 60 p = 4/3 14.0 / 12.4, 16384 x 32 k = 4 22.1 / 13.6,
-// 4000 x 200 17.4 / 12.6, 4096 x 512 17.6 / 16.0; 16384 x 64 k = 2 7.3 / 7.6); rows in whole waves do not care.
+// Newton kernel, rows read straight into registers: after the iteration.  Earlier, with rows that take unequally many passes,
+// the next grid's blocks share the SMs unevenly (forward pass, us, call after the row's loads / after the iteration: 2097 x
+// 1000 p = 2 9.0 / 7.7, a third masked 51 / 38; 524 x 4000 p = 4/3 13.0 / 9.8, masked 67 / 49; k = 2, call at the start / after
+// the iteration: 16384 x 64 6.2 / 4.9, 8192 x 128 p = 4/3 10.2 / 6.8; with the VJP behind it every step the same or faster).
+// Rows through the staging tile: after the loads, k <= 2 at the start (forward + VJP, after the iteration: 65536 x 32 14.9 / 16.0,
+// k = 2 p = 4/3 131072 x 32 27.8 / 28.5).  The register VJP: after its loads and first sums (4000 x 200 with the forward
+// pass, at the start / there: 17.4 / 12.6).
 // The kernels whose blocks work long on few loads (general w, permutations, sweeps, columns, sorted rows) do not call it: the
 // next grid may start when their blocks have ended.  With it at their start, steps of a few blocks queued back to back
 // put the waiting blocks of several grids on the same few SMs (one such step: 42 us alone, 236 in a row).

@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
   const int bar = 1 + team;
   int phase = 0;                               // which of the two buffers the next team sum uses
 
-  if (KSEL != 0) overlap_next();               // k <= 2: no iteration to speak of, the next grid may queue at once
+  if (STAGED && KSEL != 0) overlap_next();     // (where the calls stand: tk_common.cuh)
   overlap_wait();
   if (STAGED) {
     // ---- stage the warp's rows (contiguous in memory) in its tile, row stride G * E
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
       asm volatile("prefetch.global.L2 [%0];" ::"l"(P.theta + first));
   }
 
-  if (KSEL == 0) overlap_next();
+  if (STAGED && KSEL == 0) overlap_next();
 
   // ---- the iteration
   int passes = 0;
@@ -692,6 +692,7 @@ __global__ void __launch_bounds__(nt_threads(W), nt_min_blocks(E, W, Q4, STAGED,
       }
     }
   }
+  if (!STAGED) overlap_next();
   const Place fin = REBUILD ? Place(P, smem, nt_tid(), nt_cta()) : at;
   nt_finish<G, E, W, Q4, STAGED, WHAT>(P, fin, S, d, wid, early, bad, phase, smem);
 }
