@@ -193,8 +193,9 @@ tk_status tk_jvp(const float *theta, const float *tangent, int64_t rows, int64_t
  * (or target == NULL) means no target for that row: loss = f, grad = y*; loss: device [rows]
  * fp32; grad: device [rows*n] fp32 (it also serves as the buffer the mask is computed in).
  * opts as for tk_fwd_ex (solver, workspace, status word, row state of the mask); every limit of
- * tk_fwd_ex in TK_MASK mode applies.  Two launches: the forward pass, then one pass over
- * (theta, y*) that reduces each row and subtracts the target.                                  */
+ * tk_fwd_ex in TK_MASK mode applies.  One launch where the threshold form serves rows of up to 32768
+ * elements (p = 2, p = 4/3); elsewhere the forward pass, then one over (theta, y*) that reduces each
+ * row and subtracts the target.                                                                  */
 tk_status tk_topk_loss(const float *theta, const int32_t *target, int64_t rows, int64_t n, int64_t k,
                        double p, double lambda, float *loss, float *grad, const tk_opts *opts,
                        tk_stream stream);
